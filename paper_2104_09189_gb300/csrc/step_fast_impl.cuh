@@ -277,6 +277,51 @@ __device__ __forceinline__ int unpack_sign(uint32_t r, int k)
     return v == 1u ? 1 : (v == 2u ? -1 : 0);
 }
 
+// Signs of the edges selected by `need` (as exact_signs) for a foot that came
+// out of the foot arithmetic as node i's own pair, in a triangle with node i
+// as a vertex.  The foot is then node i + d exactly, d = pair - double
+// coordinate (|d| <= 2^-49, exact in float for all but tiny coordinates), and
+// an edge P -> Q through node i has orient(P, Q, foot) = (Q - P) x d exactly:
+// no cancellation is left and float decides it.  With Q - P rounded from the
+// pair form (within 2^-24 relative and 2^-47 absolute of the exact
+// difference) the float cross product is within 2^-21 of the |.|-sum of its
+// products plus 2^-46 |d|_1; a sign inside that bound, or an edge not through
+// node i, stays undecided.  Returns the packed signs and, in bits 8..10, the
+// edges still undecided.  Where a field vanishes at a whole time level every
+// node comes here (the swirl's pause): with the FP64 stages of exact_signs that
+// step took 1.53 ms on 1.05 M nodes, the steps around it 0.05 ms, and a run
+// of 20 steps 2.52 ms; 1.21 ms with this.
+static __device__ __noinline__ uint32_t node_signs(const double2 *__restrict__ xyd, int i, int w0, int w1, int w2,
+                                                   float4 A, float4 B, float4 C, df X, df Y, uint32_t need)
+{
+    const double2 x = xyd[i];
+    const double ex = __dsub_rn((double)X.l, __dsub_rn(x.x, (double)X.h));    // both differences are exact
+    const double ey = __dsub_rn((double)Y.l, __dsub_rn(x.y, (double)Y.h));
+    const float dx = __double2float_rn(ex), dy = __double2float_rn(ey);
+    const float dd = fabsf(dx) + fabsf(dy);
+    // (below 2^-90 the products come near the subnormals)
+    if ((double)dx != ex || (double)dy != ey || (dd != 0.0f && dd < 0x1p-90f)) return need << 8;
+    uint32_t out = 0, left = 0;
+    for (int k = 0; k < 3; ++k) {
+        if (!(need >> k & 1u)) continue;
+        const float4 P = k == 0 ? B : (k == 1 ? C : A), Q = k == 0 ? C : (k == 1 ? A : B);
+        const int p = k == 0 ? w1 : (k == 1 ? w2 : w0), q = k == 0 ? w2 : (k == 1 ? w0 : w1);
+        if (p != i && q != i) {
+            left |= 1u << k;
+            continue;
+        }
+        const float qx = __fadd_rn(__fsub_rn(Q.x, P.x), __fsub_rn(Q.z, P.z));
+        const float qy = __fadd_rn(__fsub_rn(Q.y, P.y), __fsub_rn(Q.w, P.w));
+        const float t1 = __fmul_rn(qx, dy), t2 = __fmul_rn(qy, dx);
+        const float c = __fsub_rn(t1, t2), e = 0x1p-21f * (fabsf(t1) + fabsf(t2)) + 0x1p-46f * dd;
+        if (dd == 0.0f) continue;                    // the foot is the node: exactly 0
+        if (c > e) out |= 1u << (2 * k);
+        else if (c < -e) out |= 2u << (2 * k);
+        else left |= 1u << k;
+    }
+    return out | (left << 8);
+}
+
 // Randomised visibility walk step: a uniformly drawn negative edge (signs
 // s1..s3 of the edges opposite W0..W2, at least one negative).
 __device__ __forceinline__ int random_negative_edge(int64_t i, uint32_t hops, int s1, int s2, int s3)
@@ -722,7 +767,9 @@ struct NodeCounters {
 // test and the value always take the triangle's vertices in slot order
 // (T[0][j], T[1][j], T[2][j]), so the result depends on the located triangle
 // and the foot only, not on the path of the walk.
-template <bool kDebug, bool kExt, bool kCompact>
+//
+// kCount: the variants that count or report (statistics, debug outputs).
+template <bool kDebug, bool kCount, bool kExt, bool kCompact>
 __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, NodeCounters &c)
 {
     const FastProb &P = a.probs[pi];
@@ -901,8 +948,18 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
             if (s3 == 2) { const int32_t nb = a.tn[2][j]; if (nb < 0 && (fside >> (-1 - nb) & 1u)) s3 = 0; }
         }
         if (s1 == 2 || s2 == 2 || s3 == 2) {
+            uint32_t need = (s1 == 2 ? 1u : 0u) | (s2 == 2 ? 2u : 0u) | (s3 == 2 ? 4u : 0u);
+            if (!kCount && at_node) {
+                // the foot is the node's own pair (the counting variants take the
+                // stages below, which give the same signs)
+                const uint32_t r = node_signs(a.xyd, (int)i, w0, w1, w2, A, B, C, X, Y, need), done = need & ~(r >> 8);
+                if (done & 1u) s1 = unpack_sign(r, 0);
+                if (done & 2u) s2 = unpack_sign(r, 1);
+                if (done & 4u) s3 = unpack_sign(r, 2);
+                need &= r >> 8;
+            }
             // exact signs on the double coordinates and the exact foot
-            const uint32_t r = exact_signs(a.xyd, w0, w1, w2, X, Y, (s1 == 2 ? 1u : 0u) | (s2 == 2 ? 2u : 0u) | (s3 == 2 ? 4u : 0u));
+            const uint32_t r = need ? exact_signs(a.xyd, w0, w1, w2, X, Y, need) : 0u;
             if (s1 == 2) s1 = unpack_sign(r, 0);
             if (s2 == 2) s2 = unpack_sign(r, 1);
             if (s3 == 2) s3 = unpack_sign(r, 2);
@@ -1008,7 +1065,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_step_fast_df(FastArgs a)
     // level (a level mixes problems)
     const int pi = !active || a.nprob == 1 ? 0
                    : (kExt && a.order ? problem_of(a.node_off, a.nprob, i) : chunk_problem(a.chunk_prob, a.node_off, i));
-    if (active) step_node<kDebug, kExt, kCompact>(a, i, pi, c);
+    if (active) step_node<kDebug, kStats || kDebug, kExt, kCompact>(a, i, pi, c);
     if (kStats) warp_stats(a.stats, active, c.hops, c.exact, c.clipped, c.fallback, c.limit, c.filter2, c.excluded);
 }
 
@@ -1158,7 +1215,7 @@ __global__ void __launch_bounds__(128, 8) k_finish_df(FastArgs a)
     for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < count; q += gridDim.x * blockDim.x) {
         NodeCounters c;
         const int64_t i = a.queue[q];
-        step_node<kDebug, false, kCompact>(a, i, a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i), c);
+        step_node<kDebug, kStats || kDebug, false, kCompact>(a, i, a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i), c);
         tot.hops += c.hops;
         hmax = c.hops > hmax ? c.hops : hmax;
         tot.exact += c.exact;
