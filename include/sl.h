@@ -126,7 +126,11 @@ typedef struct {
 /* Tunable options (sl_mesh_set_option) */
 typedef enum {
     SL_OPT_STATS = 0,        /* 0/1: accumulate sl_stats counters (default 0) */
-    SL_OPT_WALK_CAP = 1,     /* hops before the fallback rule (default max(64, 4 (M+1))) */
+    SL_OPT_WALK_CAP = 1,     /* hops before the fallback rule (0 = default: max(64, 4 (M+1))).  With the
+                                default cap and strategy (b), a step that neither counts nor
+                                reports (no statistics, no debug outputs) may start a long walk
+                                at a table of start triangles nearer the foot; the located
+                                triangles and values are those of the walk from T^0. */
     SL_OPT_KERNEL = 2,       /* 0 = auto (fast), 1 = plain FP64 kernel, 2 = fast kernel */
     SL_OPT_BLOCK = 3,        /* threads per block of the plain FP64 kernel (0 = auto) */
     /* 4 and 6 are not options (SL_E_ARG) */

@@ -111,7 +111,7 @@ void free_device(sl_mesh *m)
     release_l2_window(m);
     DeviceMesh &d = m->d;
     void *ptrs[] = {d.xy, d.tv[0], d.tv[1], d.tv[2], d.tn[0], d.tn[1], d.tn[2], d.t0, d.t0_init, d.t0v, d.node_off, d.chunk_prob,
-                    d.status, d.stats, d.probs, d.fprobs, d.xyq, d.xyh, d.g1, d.g2, d.tparams, d.dfa, d.dfb, d.he, d.he8, d.grid_t0v, d.tree_order, d.tree_parent, d.queue, d.queue_count,
+                    d.status, d.stats, d.probs, d.fprobs, d.xyq, d.xyh, d.g1, d.g2, d.tparams, d.dfa, d.dfb, d.he, d.he8, d.tri, d.jump, d.grid_t0v, d.tree_order, d.tree_parent, d.queue, d.queue_count,
                     m->host_v, m->host_v2};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -142,6 +142,8 @@ static float hop_edge_bound(const sl_mesh *m, const std::vector<float2> &h)
     const float f = (float)L;
     return (double)f >= L ? f : std::nextafter(f, __builtin_inff());
 }
+
+static sl_status build_jump_table(sl_mesh *m);
 
 // Copy the host arrays (current numbering) to the device, converting local
 // indices to global ones.
@@ -199,6 +201,8 @@ static sl_status upload_arrays(sl_mesh *m)
     // half-edge walk records of the fast kernels
     sl_status st = build_walk_records(m);
     if (st != SL_OK) return st;
+    launch_build_tri(d.tv, Nt, (int4 *)d.tri, 0);
+    SL_CUDA(cudaGetLastError());
     SL_CUDA(cudaMemcpy(d.t0, m->t0.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice));
     SL_CUDA(cudaMemcpy(d.t0_init, m->t0_init.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice));
     SL_CUDA(cudaMemcpy(d.node_off, m->node_off.data(), sizeof(int64_t) * (m->n_problems + 1), cudaMemcpyHostToDevice));
@@ -217,9 +221,60 @@ static sl_status upload_arrays(sl_mesh *m)
         if (!d.chunk_prob) SL_CUDA(cudaMalloc(&d.chunk_prob, sizeof(int2) * nc));
         SL_CUDA(cudaMemcpy(d.chunk_prob, cp.data(), sizeof(int2) * nc, cudaMemcpyHostToDevice));
     }
+    st = build_jump_table(m);
+    if (st != SL_OK) return st;
     launch_fill_t0v(d.t0, d.tv[0], d.tv[1], d.tv[2], (int4 *)d.t0v, N, 0);
     SL_CUDA(cudaGetLastError());
     SL_CUDA(cudaDeviceSynchronize());
+    return SL_OK;
+}
+
+// The jump table of every problem: a grid of about one cell per four nodes,
+// built on the device (its scratch is the start-state cache, 16 bytes per
+// node, filled afterwards: 2 bytes per node of seeds and two integers per
+// problem of at least 3 nodes).
+static sl_status build_jump_table(sl_mesh *m)
+{
+    DeviceMesh &d = m->d;
+    const int32_t np = m->n_problems;
+    m->jump_g.resize(np);
+    m->jump_off.resize(np + 1);
+    int64_t cells = 0;
+    int32_t max_g = 1;
+    for (int32_t p = 0; p < np; ++p) {
+        const double n = (double)(m->node_off[p + 1] - m->node_off[p]);
+        const int32_t g = std::max(1, (int32_t)(0.5 * std::sqrt(n)));
+        m->jump_g[p] = g;
+        m->jump_off[p] = (int32_t)cells;
+        cells += (int64_t)g * g;
+        max_g = std::max(max_g, g);
+    }
+    m->jump_off[np] = (int32_t)cells;     // at most a quarter of the nodes: an int32
+    if (!d.jump) SL_CUDA(cudaMalloc(&d.jump, sizeof(int4) * (size_t)cells));
+    uint32_t *seed = (uint32_t *)d.t0v;
+    int32_t *off = (int32_t *)(seed + 2 * (size_t)cells);
+    std::vector<int32_t> hg(m->jump_off);
+    hg.insert(hg.end(), m->jump_g.begin(), m->jump_g.end());
+    SL_CUDA(cudaMemcpy(off, hg.data(), sizeof(int32_t) * hg.size(), cudaMemcpyHostToDevice));
+    JumpBuildArgs a;
+    for (int k = 0; k < 3; ++k) {
+        a.tv[k] = d.tv[k];
+        a.tn[k] = d.tn[k];
+    }
+    a.xyc = m->precision == SL_FP64 ? (const float2 *)d.xyh : (const float2 *)d.xy;
+    a.t0_init = d.t0_init;
+    a.node_off = d.node_off;
+    a.off = off;
+    a.gp = off + np + 1;
+    a.nprob = np;
+    a.cells = (int32_t)cells;
+    a.max_g = max_g;
+    a.N = m->N;
+    a.seed[0] = seed;
+    a.seed[1] = a.seed[0] + cells;
+    a.jump = (int4 *)d.jump;
+    launch_build_jump(a, 0);
+    SL_CUDA(cudaGetLastError());
     return SL_OK;
 }
 
@@ -270,6 +325,7 @@ sl_status upload(sl_mesh *m)
         SL_CUDA(cudaMalloc(&d.tv[k], sizeof(int32_t) * Nt));
         SL_CUDA(cudaMalloc(&d.tn[k], sizeof(int32_t) * Nt));
     }
+    SL_CUDA(cudaMalloc(&d.tri, sizeof(int4) * (Nt > 0 ? Nt : 1)));
     SL_CUDA(cudaMalloc(&d.t0, sizeof(int32_t) * N));
     if (m->precision == SL_FP64) SL_CUDA(cudaMalloc(&d.xyh, sizeof(float2) * N));
     SL_CUDA(cudaMalloc(&d.t0_init, sizeof(int32_t) * N));
@@ -377,8 +433,14 @@ FastArgs make_fast_args(const sl_mesh *m, const FastProb *fp, const void *vin, v
         a.tv[k] = m->d.tv[k];
         a.tn[k] = m->d.tn[k];
     }
+    a.tri = (const int4 *)m->d.tri;
     a.he = (const float4 *)m->d.he;
     a.he8 = (const uint2 *)m->d.he8;
+    // strategy (b) with the default hop cap may start a far walk at the jump
+    // table; the other strategies and a cap set by the caller are about the
+    // walk itself
+    a.jump = m->opt_strategy == 0 && m->opt_walk_cap == 0 ? (const int4 *)m->d.jump : nullptr;
+    a.t0_init = m->d.t0_init;
     a.t0 = m->d.t0;
     a.t0v = (int4 *)m->d.t0v;
     a.vin = vin;
@@ -420,12 +482,13 @@ FastArgs make_fast_args(const sl_mesh *m, const FastProb *fp, const void *vin, v
 static bool use_fast(const sl_mesh *m) { return m->opt_kernel != 1 || m->precision == SL_FP32; }
 
 // Per-step constants of the fast kernels (see FastProb), of one problem.
-static void fill_fast_one(const ProbStep &q, FastProb &f)
+static void fill_fast_one(const sl_mesh *m, int32_t p, const ProbStep &q, FastProb &f)
 {
     const double pi = 3.14159265358979323846;
     std::memset(&f, 0, sizeof(f));
     f.kind = q.kind;
-    f.dt = q.dt;
+    f.jump_g = m->jump_g[p];
+    f.jump_off = m->jump_off[p];
     double c[6] = {0, 0, 0, 0, 0, 0};
     switch (q.kind) {
     case SL_FIELD_AFFINE:
@@ -457,15 +520,15 @@ static void fill_fast_one(const ProbStep &q, FastProb &f)
 
 static void fill_fast(const sl_mesh *m, const ProbStep *ps, FastProb *out)
 {
-    for (int32_t p = 0; p < m->n_problems; ++p) fill_fast_one(ps[p], out[p]);
+    for (int32_t p = 0; p < m->n_problems; ++p) fill_fast_one(m, p, ps[p], out[p]);
 }
 
-sl_status fast_constants_one(const sl_problem &q, int64_t n, int32_t p, FastProb &f)
+sl_status fast_constants_one(const sl_mesh *m, const sl_problem &q, int64_t n, int32_t p, FastProb &f)
 {
     ProbStep s;
     const sl_status st = fill_step_one(q, n, p, s);
     if (st != SL_OK) return st;
-    fill_fast_one(s, f);
+    fill_fast_one(m, p, s, f);
     return SL_OK;
 }
 

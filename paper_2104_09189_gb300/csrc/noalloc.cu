@@ -128,7 +128,7 @@ extern "C" sl_status sl_step_noalloc(sl_mesh *m, const sl_problem *probs, int64_
 
     FastProb host[kNoAllocMaxProblems];
     for (int32_t p = 0; p < m->n_problems; ++p) {
-        st = fast_constants_one(probs[p], n, p, host[p]);
+        st = fast_constants_one(m, probs[p], n, p, host[p]);
         if (st != SL_OK) return st;
     }
     cudaStream_t s = (cudaStream_t)stream;

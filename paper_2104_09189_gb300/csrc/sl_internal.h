@@ -54,6 +54,8 @@ struct DeviceMesh {
     double *tparams = nullptr;        // field parameters the tables were built from (device)
     void *dfa = nullptr, *dfb = nullptr;   // value scratch of sl_step for the fast FP64 kernel
     void *he = nullptr;               // float4 half-edge walk records of the fast kernels (3 Nt), or NULL
+    void *tri = nullptr;              // int4 (3 t, its vertex ids) per triangle
+    void *jump = nullptr;             // int4 start state per cell of the problems' jump tables
     void *he8 = nullptr;              // uint2 compact records (FP64 meshes that fit, 3 Nt), or NULL
 };
 
@@ -84,6 +86,7 @@ struct sl_mesh {
     std::vector<int32_t> tri, nbr;
     std::vector<int32_t> t0;          // T^0, global triangle indices (host copy)
     std::vector<int32_t> t0_init;     // the initial T^0 chosen at creation
+    std::vector<int32_t> jump_g, jump_off;   // per problem: cells per side and first cell of its jump table
     std::vector<int32_t> cells;       // per problem: sqrt(Nt/2), the M of a grid mesh
     // options
     int32_t opt_stats = 0;
@@ -141,7 +144,7 @@ sl_status build_walk_records(sl_mesh *m);
 // give back the persisting L2 lines and the context's previous limit
 void release_l2_window(sl_mesh *m);
 // the fast kernels' constants of step n of one problem, validated as sl_step validates them
-sl_status fast_constants_one(const sl_problem &q, int64_t n, int32_t p, FastProb &f);
+sl_status fast_constants_one(const sl_mesh *m, const sl_problem &q, int64_t n, int32_t p, FastProb &f);
 // the arguments of a fast-kernel step of the whole mesh: the step's constants
 // on the device (fp) and on the host (fh, or NULL; a single problem's are
 // also passed in the kernel parameters), values vin -> vout, debug outputs

@@ -153,4 +153,7 @@ __device__ __forceinline__ int chunk_problem(const int2 *chunk_prob, const int64
     return c.x + problem_of(node_off + c.x, c.y - c.x + 1, i);
 }
 
+// Cell of a coordinate on a grid of g cells over [0, 1].
+__device__ __forceinline__ int jump_cell(float x, int g) { return min(max((int)(x * (float)g), 0), g - 1); }
+
 }  // namespace sl

@@ -75,20 +75,26 @@ void launch_finish_df(const FastArgs &a, bool stats, bool debug, int sms, cudaSt
 // register budget is sized for): 0 = 256 x 4 (64 registers), 1 = 256 x 3,
 // 2 = 128 x 8, 3 = 128 x 9 (56 registers), 4 = 256 x 5, 5 = 128 x 12.  Each
 // is instantiated in a translation unit of its own pair (step_fast_c*.cu).
+//
+// They are configurations of the lean kernel.  Statistics, debug outputs and
+// strategy (c) run the full node step in one configuration of its own.
 void launch_fast_df(const FastArgs &a, bool stats, bool debug, int config, cudaStream_t s)
 {
-    if (a.exclude || a.order || a.grid_M > 0 || a.keep_t0) {
-        // the experiment options: one configuration (128 x 8, 64 registers)
-        launch_fast_df_ext(a, stats, debug, s);
+    if (stats || debug || a.order) {
+        launch_full_df(a, stats, debug, s);
+        return;
+    }
+    if (a.exclude || a.grid_M > 0 || a.keep_t0) {
+        launch_lean_df_ext(a, s);
         return;
     }
     switch (config) {
-    case 1: launch_fast_df_c1(a, stats, debug, s); break;
-    case 2: launch_fast_df_c2(a, stats, debug, s); break;
-    case 3: launch_fast_df_c3(a, stats, debug, s); break;
-    case 4: launch_fast_df_c4(a, stats, debug, s); break;
-    case 5: launch_fast_df_c5(a, stats, debug, s); break;
-    default: launch_fast_df_c0(a, stats, debug, s); break;
+    case 1: launch_lean_df_c1(a, s); break;
+    case 2: launch_lean_df_c2(a, s); break;
+    case 3: launch_lean_df_c3(a, s); break;
+    case 4: launch_lean_df_c4(a, s); break;
+    case 5: launch_lean_df_c5(a, s); break;
+    default: launch_lean_df_c0(a, s); break;
     }
 }
 
@@ -290,6 +296,95 @@ __global__ void k_fill_t0v(const int32_t *__restrict__ t0, const int32_t *__rest
     }
 }
 
+// Jump table, pass 1: the least initial triangle of the nodes in each cell.
+__global__ void k_jump_seed(JumpBuildArgs a)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.N; i += (int64_t)gridDim.x * blockDim.x) {
+        const int p = a.nprob == 1 ? 0 : problem_of(a.node_off, a.nprob, i);
+        const int g = a.gp[p];
+        const float2 x = a.xyc[i];
+        atomicMin(&a.seed[0][a.off[p] + jump_cell(x.y, g) * g + jump_cell(x.x, g)], (uint32_t)a.t0_init[i]);
+    }
+}
+
+// The problem of a cell (binary search over the cell offsets).
+__device__ __forceinline__ int jump_problem(const int32_t *off, int nprob, int32_t c)
+{
+    int lo = 0, hi = nprob;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (off[mid] <= c) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// Pass 2, with r = 1, 2, 4, ...: a cell without a seed takes the least seed of
+// the cells r away in the eight directions (any triangle will do; it should be
+// near).
+__global__ void k_jump_fill(JumpBuildArgs a, int r, int from)
+{
+    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < a.cells; c += gridDim.x * blockDim.x) {
+        uint32_t v = a.seed[from][c];
+        if (v == 0xFFFFFFFFu) {
+            const int p = a.nprob == 1 ? 0 : jump_problem(a.off, a.nprob, c);
+            const int g = a.gp[p], q = c - a.off[p], m = q / g, l = q - m * g;
+            for (int dm = -r; dm <= r; dm += r)
+                for (int dl = -r; dl <= r; dl += r)
+                    if (m + dm >= 0 && m + dm < g && l + dl >= 0 && l + dl < g)
+                        v = min(v, a.seed[from][a.off[p] + (m + dm) * g + l + dl]);
+        }
+        a.seed[from ^ 1][c] = v;
+    }
+}
+
+// Pass 3: from the seed triangle, cross the edge the cell's centre lies
+// furthest beyond, at most 64 times (float: any triangle is a valid start).
+// A cell that found no seed takes triangle of its problem's first node.
+__global__ void k_jump_walk(JumpBuildArgs a, int from)
+{
+    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < a.cells; c += gridDim.x * blockDim.x) {
+        const int p = a.nprob == 1 ? 0 : jump_problem(a.off, a.nprob, c);
+        const int g = a.gp[p], q = c - a.off[p], m = q / g, l = q - m * g;
+        const float X = ((float)l + 0.5f) / (float)g, Y = ((float)m + 0.5f) / (float)g;
+        const uint32_t seed = a.seed[from][c];
+        int32_t j = seed == 0xFFFFFFFFu ? a.t0_init[a.node_off[p]] : (int32_t)seed;
+        int w[3];
+        for (int hop = 0;; ++hop) {
+            float2 V[3];
+            for (int k = 0; k < 3; ++k) {
+                w[k] = a.tv[k][j];
+                V[k] = a.xyc[w[k]];
+            }
+            float best = 0.0f;
+            int b = -1;
+            for (int k = 0; k < 3; ++k) {
+                const float2 A = V[(k + 1) % 3], B = V[(k + 2) % 3];
+                const float o = (A.x - X) * (B.y - Y) - (A.y - Y) * (B.x - X);
+                if (o < best) {
+                    best = o;
+                    b = k;
+                }
+            }
+            if (b < 0 || hop == 64) break;
+            const int32_t u = a.tn[b][j];
+            if (u < 0) break;
+            j = u;
+        }
+        a.jump[c] = make_int4(3 * j, w[0], w[1], w[2]);
+    }
+}
+
+void launch_build_jump(const JumpBuildArgs &a, cudaStream_t s)
+{
+    if (a.N <= 0 || a.cells <= 0) return;
+    cudaMemsetAsync(a.seed[0], 0xFF, sizeof(uint32_t) * (size_t)a.cells, s);
+    k_jump_seed<<<grid_for(a.N, 256), 256, 0, s>>>(a);
+    int from = 0;
+    for (int r = 1; r < 2 * a.max_g; r *= 2, from ^= 1) k_jump_fill<<<grid_for(a.cells, 256), 256, 0, s>>>(a, r, from);
+    k_jump_walk<<<grid_for(a.cells, 128), 128, 0, s>>>(a, from);
+}
+
 struct HalfEdgeArgs {
     const int32_t *tv[3];
     const int32_t *tn[3];
@@ -388,6 +483,18 @@ void launch_build_he8(const int32_t *const tv[3], const int32_t *const tn[3], co
     a.he8 = he8;
     a.overflow = overflow;
     if (nt > 0) k_build_he8<<<grid_for(3 * nt, 256), 256, 0, s>>>(a);
+}
+
+__global__ void k_build_tri(const int32_t *__restrict__ tv0, const int32_t *__restrict__ tv1,
+                            const int32_t *__restrict__ tv2, int4 *__restrict__ tri, int64_t nt)
+{
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += (int64_t)gridDim.x * blockDim.x)
+        tri[t] = make_int4(3 * (int32_t)t, tv0[t], tv1[t], tv2[t]);
+}
+
+void launch_build_tri(const int32_t *const tv[3], int64_t nt, int4 *tri, cudaStream_t s)
+{
+    if (nt > 0) k_build_tri<<<grid_for(nt, 256), 256, 0, s>>>(tv[0], tv[1], tv[2], tri, nt);
 }
 
 void launch_fill_t0v(const int32_t *t0, const int32_t *tv0, const int32_t *tv1, const int32_t *tv2, int4 *t0v,

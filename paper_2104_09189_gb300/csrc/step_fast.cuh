@@ -6,6 +6,7 @@
 #include <cstdint>
 
 #include "../../include/sl.h"
+#include "step_common.cuh"
 
 namespace sl {
 
@@ -25,7 +26,8 @@ namespace sl {
 struct FastProb {
     int32_t kind;
     int32_t flags;      // kFastCentreGrid
-    double dt;          // only used by the clip path and the debug output
+    int32_t jump_g;     // cells per side of the problem's jump table
+    int32_t jump_off;   // its first cell in FastArgs::jump
     float2 c[6];        // (hi, lo)
 };
 
@@ -43,8 +45,14 @@ struct FastArgs {
     const float2 *xyh;            // FP64 meshes: high parts (xh, yh) for the FP32 hop tests
     const int32_t *tv[3];
     const int32_t *tn[3];         // -1 - side on the boundary (0: x=0, 1: x=1, 2: y=0, 3: y=1)
+    const int4 *tri;              // per triangle: (3 t, its three vertex ids), the start state of t
     const float4 *he;             // half-edge walk records, 3 per triangle (k_build_he), or NULL
     const uint2 *he8;             // FP64 meshes whose records fit in 8 bytes (k_build_he8), or NULL
+    // Start states (as t0v) of a triangle in or near each cell of a uniform
+    // grid over the square, per problem (FastProb::jump_off, jump_g); NULL: walks
+    // start at T^0 only
+    const int4 *jump;
+    const int32_t *t0_init;       // the node's initial incident triangle
     int32_t *t0;
     int4 *t0v;                    // per node: (3 T^0, T[0][T^0], T[1][T^0], T[2][T^0]), kept in
                                   // step with t0
@@ -102,6 +110,37 @@ struct FastArgs {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// The jump table (launch_build_jump).  jump_far: the foot, (dx, dy) from a
+// vertex of a triangle that does not hold it, is more than kJumpFar cells
+// away, so that the table's triangle is surely nearer.  A walk makes about two
+// hops per cell of the mesh, a cell of the table is two of the mesh wide, and
+// a jump costs two dependent gathers before its one or two hops: with 1, 2, 4
+// and 8 cells a study run of 150 k nodes with 4 hops per node took 422, 389,
+// 384 and 448 us, an FP32 swirl on 4.2 M nodes with 20 to 40 hops 3.17, 3.14,
+// 3.25 and 3.72 ms, and shorter walks stayed level from 2 on.  Four times the
+// cells gained 2 % there and nothing elsewhere.  From the initial triangles, a
+// rotation 360 cells long on 16.8 M nodes: 16.8 ms per run of 50 steps by
+// walking, 9.6 ms with the table (its first step 8.0 -> 0.7 ms).
+constexpr float kJumpFar = 3.0f;
+__device__ __forceinline__ bool jump_far(float dx, float dy, const FastProb &P)
+{
+    return (fabsf(dx) + fabsf(dy)) * (float)P.jump_g > kJumpFar;
+}
+__device__ __forceinline__ int4 jump_start(const FastArgs &a, const FastProb &P, float x, float y)
+{
+    const int g = P.jump_g;
+    return __ldg(&a.jump[P.jump_off + jump_cell(y, g) * g + jump_cell(x, g)]);
+}
+
+// A foot found in triangle j with these signs (none negative, at least one
+// zero) lies on a vertex or on an edge between two triangles; a zero on one
+// edge of the boundary alone leaves j the only triangle.
+__device__ __forceinline__ bool shared_zero(const FastArgs &a, int32_t j, int s1, int s2, int s3)
+{
+    if ((s1 == 0) + (s2 == 0) + (s3 == 0) > 1) return true;
+    return a.tn[s1 == 0 ? 0 : (s2 == 0 ? 1 : 2)][j] >= 0;
+}
+
 template <typename Kernel>
 inline void launch_step_kernel(Kernel k, unsigned grid, unsigned block, cudaStream_t s, const FastArgs &a)
 {
@@ -125,14 +164,16 @@ inline void launch_step_kernel(Kernel k, unsigned grid, unsigned block, cudaStre
 
 // config: launch configuration 0..kFastConfigs-1 (see step_fast.cu)
 void launch_fast_df(const FastArgs &a, bool stats, bool debug, int config, cudaStream_t s);
-// one launch configuration each (step_fast_c*.cu)
-void launch_fast_df_c0(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
-void launch_fast_df_c1(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
-void launch_fast_df_c2(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
-void launch_fast_df_c3(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
-void launch_fast_df_c4(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
-void launch_fast_df_c5(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
-void launch_fast_df_ext(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
+// one launch configuration each of the lean kernel (step_fast_c*.cu)
+void launch_lean_df_c0(const FastArgs &a, cudaStream_t s);
+void launch_lean_df_c1(const FastArgs &a, cudaStream_t s);
+void launch_lean_df_c2(const FastArgs &a, cudaStream_t s);
+void launch_lean_df_c3(const FastArgs &a, cudaStream_t s);
+void launch_lean_df_c4(const FastArgs &a, cudaStream_t s);
+void launch_lean_df_c5(const FastArgs &a, cudaStream_t s);
+void launch_lean_df_ext(const FastArgs &a, cudaStream_t s);
+// the full node step alone: statistics, debug outputs, strategy (c)
+void launch_full_df(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
 // the two passes of a split step: lean settle pass, then the finish pass over
 // its queue (reset: zero the queue counter first)
 void launch_settle_df(const FastArgs &a, bool stats, bool debug, bool reset, cudaStream_t s);
@@ -190,6 +231,28 @@ void launch_build_he(const int32_t *const tv[3], const int32_t *const tn[3], con
 // 44.7 M triangles): the mesh then keeps 16-byte records.
 void launch_build_he8(const int32_t *const tv[3], const int32_t *const tn[3], const float2 *xyh, int64_t nt,
                       uint2 *he8, uint32_t *overflow, cudaStream_t s);
+
+// The jump table of all problems: per cell of problem p (gp cells per side,
+// first cell off[p], off and gp on the device; cells in all) the start state
+// of the triangle a walk towards the cell's centre ends in, from a triangle
+// incident to a node of the cell (or of the nearest cell that has one).
+struct JumpBuildArgs {
+    const int32_t *tv[3];
+    const int32_t *tn[3];
+    const float2 *xyc;            // float coordinates (hop coordinates of FP64 meshes)
+    const int32_t *t0_init;
+    const int64_t *node_off;
+    const int32_t *off;           // nprob + 1
+    const int32_t *gp;            // nprob
+    int32_t nprob, cells, max_g;
+    int64_t N;
+    uint32_t *seed[2];            // scratch, cells each
+    int4 *jump;
+};
+void launch_build_jump(const JumpBuildArgs &a, cudaStream_t s);
+
+// tri[t] = (3 t, its three vertex ids in slot order)
+void launch_build_tri(const int32_t *const tv[3], int64_t nt, int4 *tri, cudaStream_t s);
 
 // t0v[i] = (3 t0[i], its three vertex ids in slot order)
 void launch_fill_t0v(const int32_t *t0, const int32_t *tv0, const int32_t *tv1, const int32_t *tv2, int4 *t0v,

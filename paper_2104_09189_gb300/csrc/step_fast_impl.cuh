@@ -523,10 +523,12 @@ __device__ __forceinline__ void foot_to_grid(df &X, df &Y)
 // double-float, decided against the boundary in double rounding, clipped and
 // then split.  Returns true when clipped.  at_node: a foot on or beyond a side
 // that is the node itself (an outward boundary node); a foot inside the
-// square is not reported here.
-template <int kKind>
+// square is not reported here.  gone (kExt, with a.exclude): the foot leaves
+// the square and the node is excluded (X, Y are then not set).
+// kInside: a foot inside the square that is its node's pair is reported too.
+template <int kKind, bool kExt = false, bool kInside = false>
 __device__ __forceinline__ bool foot_pair(const FastArgs &a, int64_t i, const FastProb &P, df &X, df &Y,
-                                          bool &at_node)
+                                          bool &at_node, bool &gone)
 {
     const float4 xq = a.xyq[i];
     const df x = df_make(xq.x, xq.z), y = df_make(xq.y, xq.w);
@@ -534,7 +536,11 @@ __device__ __forceinline__ bool foot_pair(const FastArgs &a, int64_t i, const Fa
     if (kKind < 0) disp_df(P, a, i, x, y, DX, DY);
     else disp_df_k<kKind < 0 ? 0 : kKind>(P, a, i, x, y, DX, DY);
     at_node = false;
-    if (foot_grid(x, DX, X) & foot_grid(y, DY, Y)) return false;
+    gone = false;
+    if (foot_grid(x, DX, X) & foot_grid(y, DY, Y)) {
+        if (kInside) at_node = foot_is_node(x, y, X, Y);
+        return false;
+    }
     X = df_add(x, DX);
     Y = df_add(y, DY);
     const bool inside = df_inside(X, Y);
@@ -542,9 +548,13 @@ __device__ __forceinline__ bool foot_pair(const FastArgs &a, int64_t i, const Fa
     if (!inside) {
         round_boundary(X);
         round_boundary(Y);
+        if (kExt && a.exclude && (df_neg_strict(X) || df_gt1(X) || df_neg_strict(Y) || df_gt1(Y))) {
+            gone = true;
+            return false;
+        }
         clipped = clip_df(x, y, X, Y);
     }
-    at_node = !inside && foot_is_node(x, y, X, Y);
+    at_node = (kInside || !inside) && foot_is_node(x, y, X, Y);
     foot_to_grid(X, Y);
     return clipped;
 }
@@ -949,7 +959,8 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
         }
         if (s1 == 2 || s2 == 2 || s3 == 2) {
             uint32_t need = (s1 == 2 ? 1u : 0u) | (s2 == 2 ? 2u : 0u) | (s3 == 2 ? 4u : 0u);
-            if (!kCount && at_node) {
+            const float4 xn = a.xyq[i];
+            if (!kCount && foot_is_node(df_make(xn.x, xn.z), df_make(xn.y, xn.w), X, Y)) {
                 // the foot is the node's own pair (the counting variants take the
                 // stages below, which give the same signs)
                 const uint32_t r = node_signs(a.xyd, (int)i, w0, w1, w2, A, B, C, X, Y, need), done = need & ~(r >> 8);
@@ -1130,8 +1141,8 @@ __device__ __forceinline__ bool settle_node(const FastArgs &a, int64_t i, int pi
 {
     const FastProb &P = kKind < 0 ? a.probs[pi] : a.prob0;
     df X, Y;
-    bool at_node;
-    const bool clipped = foot_pair<kKind>(a, i, P, X, Y, at_node);
+    bool at_node, gone;
+    const bool clipped = foot_pair<kKind>(a, i, P, X, Y, at_node, gone);
     const int4 tq = a.t0v[i];
     const float4 A = a.xyq[tq.y], B = a.xyq[tq.z], C = a.xyq[tq.w];
     // the start triangle's values are read together with its vertices, not
@@ -1253,7 +1264,8 @@ inline void launch_fast_df_form(const FastArgs &a, bool stats, bool debug, unsig
         else launch_step_kernel(k_step_fast_df<true, false, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
     } else {
         if (debug) launch_step_kernel(k_step_fast_df<false, true, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
-        else launch_step_kernel(k_step_fast_df<false, false, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
+        else if constexpr (kExt)    // strategy (c); the lean kernel takes the others
+            launch_step_kernel(k_step_fast_df<false, false, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
     }
 }
 

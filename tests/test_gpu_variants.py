@@ -54,3 +54,68 @@ def test_feet_at_their_nodes(M, records):
         want = om.step(f.kind, f.packed(), dt, n, before)[0]
         assert np.abs(g.from_dev(b) - want).max() <= REL_TOL_FP64 * np.abs(want).max()
         v = b
+
+
+FIELDS = {
+    "rotation": lambda: si.rotation_field(),
+    "swirl": lambda: si.swirl_field(),
+    "fourier8": lambda: si.fourier8_field(4),
+    "affine": lambda: si.affine_field([0.5, -0.3, 0.2, 0.1, 0.3, 0.1, 0.3, -0.1]),
+}
+
+
+@pytest.mark.parametrize("precision", [sl.SL_FP64, sl.SL_FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("field", list(FIELDS))
+@pytest.mark.parametrize("M,dt,graded", [(9, 0.31, False), (64, 0.2, True), (181, 0.011, False), (181, 0.11, True)])
+def test_walks_from_the_jump_table(M, dt, graded, field, precision):
+    """Feet up to half the square away start at the jump table (also on a mesh
+    of a few cells, in a clipped corner and along a side)."""
+    m = si.grid_mesh(M, 0.2, 5, graded=graded)
+    f = FIELDS[field]()
+    g = DeviceRun(m, f, dt, curve=sl.SL_CURVE_MORTON, precision=precision)
+    v = g.to_dev(si.gaussian(m.xy))
+    for n in range(4):
+        (a, b), (ja, jb) = step_both(g, n, v)
+        assert bool((ja == jb).all()), f"step {n}: located triangles differ"
+        assert bool((a == b).all()), f"step {n}: values differ"
+        v = b
+
+
+@pytest.mark.parametrize("precision", [sl.SL_FP64, sl.SL_FP32], ids=["fp64", "fp32"])
+def test_feet_on_edges_and_vertices(precision):
+    """On a Courant grid of 2^-k cells a dyadic translation puts every foot on a
+    vertex (whole cells) or on an edge (half cells): the triangle depends on
+    the walk's path, which must be the walk from T^0."""
+    m = si.courant_grid(32)
+    for shift in ((4.0, 6.0), (5.5, 0.0), (3.5, 3.5), (-7.0, 2.5)):
+        f = si.affine_field([shift[0] / 32, 0, 0, 0, shift[1] / 32, 0, 0, 0])
+        g = DeviceRun(m, f, 1.0, curve=sl.SL_CURVE_HILBERT, precision=precision)
+        v = g.to_dev(si.gaussian(m.xy))
+        for n in range(3):
+            (a, b), (ja, jb) = step_both(g, n, v)
+            assert bool((ja == jb).all()) and bool((a == b).all()), f"shift {shift}, step {n}"
+            v = b
+
+
+def test_jump_table_of_uneven_batch():
+    """Meshes of 9 to 10 000 nodes in one batch, each with a table of its own."""
+    import torch
+    meshes = [si.grid_mesh(M, 0.25, M) for M in (2, 99, 3, 40, 17, 5)]
+    fields = [si.swirl_field(), si.rotation_field(), si.fourier8_field(1), si.rotation_field(), si.swirl_field(),
+              si.fourier8_field(2)]
+    no, to, xy, tri = sl.pack_meshes([(m.xy, m.tri) for m in meshes])
+    probs = sl.problems([(f.kind, 0.07, f.packed()) for f in fields])
+    v0 = torch.tensor(np.concatenate([si.gaussian(m.xy) for m in meshes]), dtype=torch.float64, device="cuda")
+    got = []
+    for cap in (0, 1 << 20):       # a cap set by the caller turns the table off
+        h = sl.sl_mesh_create(no, to, xy, tri)
+        try:
+            sl.sl_mesh_set_option(h, sl.SL_OPT_WALK_CAP, cap)
+            v, w = v0.clone(), torch.empty_like(v0)
+            sl.sl_run(h, probs, 0, 6, v, w)
+            t0 = torch.empty(v.numel(), dtype=torch.int32, device="cuda")
+            sl.sl_mesh_get_t0(h, t0)
+            got.append((v, t0))
+        finally:
+            sl.sl_mesh_destroy(h)
+    assert bool((got[0][0] == got[1][0]).all()) and bool((got[0][1] == got[1][1]).all())
