@@ -296,7 +296,7 @@ sl_status sl_run(sl_mesh *m, const sl_problem *probs, int64_t n0, int32_t n_step
 sl_status sl_run_host(sl_mesh *m, const sl_problem *probs, int64_t n0, int32_t n_steps, void *v_host,
                       int32_t use_graph, sl_stats *stats, void *stream);
 
-/* Limits of sl_step_noalloc's static scratch (see below). */
+/* Limits of sl_step_noalloc (see below). */
 #define SL_NOALLOC_MAX_NODES (1 << 20)
 #define SL_NOALLOC_MAX_PROBLEMS 256
 
@@ -321,15 +321,15 @@ sl_status sl_run_host(sl_mesh *m, const sl_problem *probs, int64_t n0, int32_t n
  * already built for these exact problems by an earlier sl_step / sl_run call
  * on the mesh (that call allocates them); otherwise SL_E_STATE.
  *
- * All scratch lives in one library-owned static device array per GPU
- * (8 MiB of value pairs + 16 KiB of per-problem constants), held by every
- * GPU that loads the library until the process exits.  The step's constants
- * reach that array in the parameters of a small kernel; no host buffer of
- * the call is read after it returns.  The first call on a
+ * A batch's per-problem constants live in one library-owned static device
+ * array per GPU (16 KiB), held by every GPU that loads the library until the
+ * process exits; they reach it in the parameters of a small kernel (a single
+ * problem's are parameters of the step).  No host buffer of the call is read
+ * after it returns.  The first call on a
  * device looks up the array's device address (cudaGetSymbolAddress); make
- * that first call before any stream capture.  Every call on a device shares
- * the array and overwrites what it uses, so calls that overlap on the GPU
- * (other streams, other meshes) race on it: serialise them.  T^0 is updated
+ * that first call before any stream capture.  Every call with several problems
+ * shares the array and overwrites what it uses, so such calls that overlap on
+ * the GPU (other streams, other meshes) race on it: serialise them.  T^0 is updated
  * in place as in sl_step; device conditions are reported by sl_mesh_status.
  */
 sl_status sl_step_noalloc(sl_mesh *m, const sl_problem *probs, int64_t n, const double *v_in, double *v_out,

@@ -727,16 +727,20 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
     auto config_of = [&](int32_t k) { return (k == 0 && first_initial) ? m->opt_config_first : m->opt_config; };
     std::vector<FastProb> fh;   // the fast kernels' constants, host copy (filled when recording)
     if (!reuse) {
-        // synchronous copies: a graph recorded below may replay them later
-        SL_CUDA(cudaStreamSynchronize(s));
         if (fast) {
             fh.resize((size_t)m->n_problems * (size_t)n_steps);
             for (int32_t k = 0; k < n_steps; ++k)
                 fill_fast(m, host.data() + (size_t)k * m->n_problems, fh.data() + (size_t)k * m->n_problems);
-            sl_status st = ensure_fprobs(m, fper * n_steps);
-            if (st != SL_OK) return st;
-            SL_CUDA(cudaMemcpy(m->d.fprobs, fh.data(), fper * n_steps, cudaMemcpyHostToDevice));
+            if (m->n_problems > 1) {
+                // (a single problem's constants are kernel parameters.)  A
+                // synchronous copy: a graph recorded below may replay them later
+                SL_CUDA(cudaStreamSynchronize(s));
+                sl_status st = ensure_fprobs(m, fper * n_steps);
+                if (st != SL_OK) return st;
+                SL_CUDA(cudaMemcpy(m->d.fprobs, fh.data(), fper * n_steps, cudaMemcpyHostToDevice));
+            }
         } else {
+            SL_CUDA(cudaStreamSynchronize(s));
             sl_status st = ensure_probs(m, per * n_steps);
             if (st != SL_OK) return st;
             SL_CUDA(cudaMemcpy(m->d.probs, host.data(), per * n_steps, cudaMemcpyHostToDevice));
@@ -744,20 +748,30 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
     }
     auto enqueue = [&](cudaStream_t q) -> sl_status {
         if (fast && m->precision == SL_FP64) {
-            // values travel as (hi, lo) float pairs in the two caller buffers
-            launch_to_df((const double *)v, (float2 *)v2, m->N, q);
-            void *a = v2, *b = v;
+            // values travel as (hi, lo) float pairs in the two caller buffers; a
+            // first step reads the doubles itself and a last one writes them
+            // where the number of steps puts them on the right buffers (the
+            // passes of a split step take pairs only)
+            const bool can_in = !split_step(m, first_initial), can_out = !split_step(m, n_steps == 1 && first_initial);
+            const bool in = can_in && (n_steps % 2 == 0 || !can_out), out = can_out && in == (n_steps % 2 == 0);
+            void *a = v, *b = v2;
+            if (!in) {
+                launch_to_df((const double *)v, (float2 *)v2, m->N, q);
+                a = v2;
+                b = v;
+            }
             int32_t split_seq = 0;
             for (int32_t k = 0; k < n_steps; ++k) {
                 FastArgs args = make_fast_args(m, (const FastProb *)((char *)m->d.fprobs + fper * k), a, b, nullptr,
                                                fh.data() + (size_t)k * m->n_problems);
+                args.io = (in && k == 0 ? kIoIn : 0) | (out && k == n_steps - 1 ? kIoOut : 0);
                 sl_status st = launch_fast(m, args, false, config_of(k), k == 0 && first_initial, q, &split_seq, k > 0);
                 if (st != SL_OK) return st;
                 void *t = a;
                 a = b;
                 b = t;
             }
-            launch_from_df((const float2 *)a, (double *)v, m->N, q);
+            if (!out) launch_from_df((const float2 *)a, (double *)v, m->N, q);
             SL_CUDA(cudaGetLastError());
             return SL_OK;
         }
@@ -845,8 +859,8 @@ extern "C" sl_status sl_step(sl_mesh *m, const sl_problem *probs, int64_t n, con
     st = fill_step(m, probs, n, host.data());
     if (st != SL_OK) return st;
     const bool debug = dbg && (dbg->feet || dbg->tri || dbg->moves || dbg->flags || dbg->feet_lo);
-    m->graph.valid = false;   // the per-step buffers are overwritten
     if (!use_fast(m)) {
+        m->graph.valid = false;   // the per-step buffer is overwritten
         st = ensure_probs(m, sizeof(ProbStep) * m->n_problems);
         if (st != SL_OK) return st;
         SL_CUDA(cudaMemcpyAsync(m->d.probs, host.data(), sizeof(ProbStep) * m->n_problems, cudaMemcpyHostToDevice, s));
@@ -862,22 +876,28 @@ extern "C" sl_status sl_step(sl_mesh *m, const sl_problem *probs, int64_t n, con
     if (st != SL_OK) return st;
     std::vector<FastProb> fh(m->n_problems);
     fill_fast(m, host.data(), fh.data());
-    st = ensure_fprobs(m, sizeof(FastProb) * m->n_problems);
-    if (st != SL_OK) return st;
-    SL_CUDA(cudaMemcpyAsync(m->d.fprobs, fh.data(), sizeof(FastProb) * m->n_problems, cudaMemcpyHostToDevice, s));
-    SL_CUDA(cudaStreamSynchronize(s));
-    if (m->precision == SL_FP64) {
-        // double values in and out; the kernel works on (hi, lo) float pairs
+    if (m->n_problems > 1) {
+        // in the parameters of a small kernel, so that no host buffer outlives
+        // the call and nothing waits (a single problem's are parameters of the
+        // step itself)
+        m->graph.valid = false;   // the per-step buffer is overwritten
+        st = ensure_fprobs(m, sizeof(FastProb) * m->n_problems);
+        if (st != SL_OK) return st;
+        launch_put_constants(fh.data(), m->n_problems, (FastProb *)m->d.fprobs, s);
+    }
+    if (m->precision == SL_FP64 && split_step(m, m->t0_initial)) {
+        // double values in and out; a split step works on (hi, lo) float pairs
         if (!m->d.dfa) SL_CUDA(cudaMalloc(&m->d.dfa, sizeof(float2) * m->N));
         if (!m->d.dfb) SL_CUDA(cudaMalloc(&m->d.dfb, sizeof(float2) * m->N));
         launch_to_df((const double *)v_in, (float2 *)m->d.dfa, m->N, s);
         FastArgs a = make_fast_args(m, (const FastProb *)m->d.fprobs, m->d.dfa, m->d.dfb, dbg, fh.data());
-        st = launch_fast(m, a, debug, m->t0_initial ? m->opt_config_first : m->opt_config, m->t0_initial, s);
+        st = launch_fast(m, a, debug, m->opt_config, false, s);
         if (st != SL_OK) return st;
         launch_from_df((const float2 *)m->d.dfb, (double *)v_out, m->N, s);
         SL_CUDA(cudaGetLastError());
     } else {
         FastArgs a = make_fast_args(m, (const FastProb *)m->d.fprobs, v_in, v_out, dbg, fh.data());
+        if (m->precision == SL_FP64) a.io = kIoIn | kIoOut;
         st = launch_fast(m, a, debug, m->t0_initial ? m->opt_config_first : m->opt_config, m->t0_initial, s);
         if (st != SL_OK) return st;
     }

@@ -1,6 +1,8 @@
 // step_fast.cu -- the fast FP64-accuracy step kernel for GB300: launchers of
 // the split step, the gather probe, value conversions, field tables and
 // the walk records (the step kernels themselves are in step_fast_impl.cuh).
+#include <cstring>
+
 #include "step_fast_impl.cuh"
 
 namespace sl {
@@ -125,73 +127,18 @@ void launch_gather_probe(const float4 *xyq, const int4 *t0v, const float2 *vin, 
 // ---------------------------------------------------------------------------
 // Value format conversions (once per run, not per step)
 
-// h = v rounded to the nearest float (ties to even) and l = v - h rounded
-// to the nearest float, from the bits of v with integer operations, for
-// 2^-74 <= |v| < 2^127 (both parts normal floats); false otherwise.  The
-// 29 mantissa bits below the float's 23 decide the rounding of h; v - h is
-// then the signed integer rem (or rem - 2^29) times 2^(e - 1075), exact, and
-// converting that integer to float rounds it once, the scaling by a power of
-// two being exact in the normal range.  GB300 converts double to float on its
-// slow FP64 pipe, so this keeps the conversion at memory speed.
-__device__ __forceinline__ bool split_double_bits(double v, float &h, float &l)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
-    const int e = (int)((hi >> 20) & 0x7FFu);
-    if (e < 1075 - 126 || e > 1023 + 126) return false;
-    const uint32_t sign = hi & 0x80000000u;
-    const uint32_t top = ((hi & 0xFFFFFu) << 3) | (lo >> 29);   // the float's 23 mantissa bits
-    const uint32_t rem = lo & 0x1FFFFFFFu;                       // the 29 bits below them
-    const bool up = rem > 0x10000000u || (rem == 0x10000000u && (top & 1u));
-    const uint32_t fb = (((uint32_t)(e - 1023 + 127) << 23) | top) + (up ? 1u : 0u);   // a carry bumps the exponent
-    h = __uint_as_float(sign | fb);
-    const int32_t r = up ? (int32_t)rem - 0x20000000 : (int32_t)rem;
-    const float scale = __uint_as_float((uint32_t)(e - 1075 + 127) << 23);   // 2^(e - 1075)
-    const float m = __fmul_rn(__int2float_rn(r), scale);
-    l = sign ? -m : m;
-    return true;
-}
-
 __global__ void k_to_df(const double *__restrict__ src, float2 *__restrict__ dst, int64_t n)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double v = src[i];
-        float h, l;
-        if (!split_double_bits(v, h, l)) {
-            // zero, tiny, huge or not finite: the FP64 pipe
-            h = __double2float_rn(v);
-            l = __double2float_rn(v - (double)h);
-        }
-        dst[i] = make_float2(h, l);
+        dst[i] = pair_of_double(src[i]);
     }
-}
-
-// A float as a double from its bits (exact) for zero and normal floats;
-// false for subnormal, infinite and NaN ones.
-__device__ __forceinline__ bool widen_float_bits(float f, double &d)
-{
-    const uint32_t u = __float_as_uint(f);
-    const uint32_t ef = (u >> 23) & 0xFFu;
-    const unsigned long long sign = (unsigned long long)(u & 0x80000000u) << 32;
-    if ((u & 0x7FFFFFFFu) == 0u) {
-        d = __longlong_as_double((long long)sign);
-        return true;
-    }
-    if (ef == 0u || ef == 0xFFu) return false;
-    d = __longlong_as_double((long long)(sign | ((unsigned long long)(ef - 127u + 1023u) << 52) |
-                                         ((unsigned long long)(u & 0x7FFFFFu) << 29)));
-    return true;
 }
 
 __global__ void k_from_df(const float2 *src, double *dst, int64_t n)
 {
     // may run in place (src and dst alias, same 8-byte slots)
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float2 v = src[i];
-        double a, b;
-        if (!widen_float_bits(v.x, a)) a = (double)v.x;
-        if (!widen_float_bits(v.y, b)) b = (double)v.y;
-        dst[i] = a + b;
+        dst[i] = double_of_pair(src[i]);
     }
 }
 
@@ -210,6 +157,31 @@ void launch_to_df(const double *src, float2 *dst, int64_t n, cudaStream_t s)
 void launch_from_df(const float2 *src, double *dst, int64_t n, cudaStream_t s)
 {
     if (n > 0) k_from_df<<<grid_for(n, 256), 256, 0, s>>>(src, dst, n);
+}
+
+namespace {
+constexpr int kConstChunk = 63;     // 4 KiB of parameters
+struct ConstChunk {
+    FastProb *dst;
+    int32_t count;
+    FastProb p[kConstChunk];
+};
+__global__ void k_put_constants(const __grid_constant__ ConstChunk c)
+{
+    const int t = threadIdx.x;
+    if (t < c.count) c.dst[t] = c.p[t];
+}
+}  // namespace
+
+void launch_put_constants(const FastProb *src, int32_t n, FastProb *dst, cudaStream_t s)
+{
+    for (int32_t b = 0; b < n; b += kConstChunk) {
+        ConstChunk c;
+        c.dst = dst + b;
+        c.count = n - b < kConstChunk ? n - b : kConstChunk;
+        std::memcpy(c.p, src + b, sizeof(FastProb) * (size_t)c.count);
+        k_put_constants<<<1, kConstChunk, 0, s>>>(c);
+    }
 }
 
 // ---------------------------------------------------------------------------

@@ -32,6 +32,7 @@ struct FastProb {
 };
 
 constexpr int32_t kFastCentreGrid = 1;
+constexpr int32_t kIoIn = 1, kIoOut = 2;
 
 // The six per-step constants of a problem as float pairs: (hi, lo), or for a
 // rotation centre in [0, 1]^2 the (grid, remainder) split of the node
@@ -56,8 +57,10 @@ struct FastArgs {
     int32_t *t0;
     int4 *t0v;                    // per node: (3 T^0, T[0][T^0], T[1][T^0], T[2][T^0]), kept in
                                   // step with t0
-    const void *vin;              // FP64: float2 (hi, lo) values; FP32: float values
+    const void *vin;              // FP64: float2 (hi, lo) values, or the doubles (io); FP32: float values
     void *vout;
+    int32_t io;                   // FP64: kIoIn: vin holds doubles; kIoOut: vout takes doubles.  Not in the
+                                  // passes of a split step.
     const float4 *g1, *g2;        // field tables (hi, lo) per node (FP64 meshes), or NULL
     const float2 *g1f, *g2f;      // field tables rounded to float (FP32 meshes), or NULL
     const FastProb *probs;
@@ -184,6 +187,11 @@ void launch_fast_f32(const FastArgs &a, bool stats, bool debug, int config, cuda
 // the memory accesses of a steady step with no arithmetic (sl_probe_gather)
 void launch_gather_probe(const float4 *xyq, const int4 *t0v, const float2 *vin, float2 *vout, int64_t N,
                          cudaStream_t s);
+
+// n per-problem constants (host) to dst (device) in the parameters of a small
+// kernel, 63 per launch: dst is written in stream order and src is not read
+// after the call
+void launch_put_constants(const FastProb *src, int32_t n, FastProb *dst, cudaStream_t s);
 
 // value format conversions for the double-float kernel
 void launch_to_df(const double *src, float2 *dst, int64_t n, cudaStream_t s);

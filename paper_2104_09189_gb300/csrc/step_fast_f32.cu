@@ -103,7 +103,7 @@ struct CountersF32 {
 template <bool kDebug, bool kExt>
 __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int pi, CountersF32 &c)
 {
-    const FastProb &P = a.probs[pi];
+    const FastProb &P = a.single ? a.prob0 : a.probs[pi];
     const float2 xf = a.xyf[i];
     float X, Y;
     foot_f32(P, a, i, xf.x, xf.y, X, Y);
@@ -369,7 +369,7 @@ __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int 
 
 // The full node step for every node: statistics, debug outputs, strategy (c).
 template <bool kStats, bool kDebug, int kBlock, int kMinBlocks, bool kExt>
-__global__ void __launch_bounds__(kBlock, kMinBlocks) k_step_fast_f32(FastArgs a)
+__global__ void __launch_bounds__(kBlock, kMinBlocks) k_step_fast_f32(const __grid_constant__ FastArgs a)
 {
     const int64_t i = kExt ? node_of_thread(a) : (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = kExt ? i >= 0 : i < a.N;

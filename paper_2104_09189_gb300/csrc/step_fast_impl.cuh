@@ -388,6 +388,35 @@ __device__ __forceinline__ Certified certify(float4 A, float4 B, float4 C, float
     return certify_bounds(numerators(A, B, C, Xg, Xr, Yg, Yr));
 }
 
+// Values in and out: the first step of a run reads the caller's doubles and
+// its last one writes them (FastArgs::io), the steps between pass (hi, lo)
+// pairs on; both are 8 bytes per node, so only the conversion of what was read
+// depends on it, about 45 instructions in two uniform branches.  A pass of its
+// own each way took 4 to 5 us beside a step of 15 us on 491 k nodes, and the
+// copy of the step's constants and the wait for it another 14: eight single
+// steps 318 -> 174 us, most of the step's own time now.
+__device__ __forceinline__ void pair_in(const FastArgs &a, float2 &v)
+{
+    if (a.io & kIoIn) v = pair_of_double(__hiloint2double(__float_as_int(v.y), __float_as_int(v.x)));
+}
+
+__device__ __forceinline__ void put_value(const FastArgs &a, int64_t i, float2 v)
+{
+    if (a.io & kIoOut) {
+        const double d = double_of_pair(v);
+        v = make_float2(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)));
+    }
+    ((float2 *)a.vout)[i] = v;
+}
+
+// V^{n+1}_i = V^n_i
+__device__ __forceinline__ void keep_value(const FastArgs &a, int64_t i)
+{
+    float2 v = ((const float2 *)a.vin)[i];
+    pair_in(a, v);
+    put_value(a, i, v);
+}
+
 // 1 / d to about 2^-24 relative: the hardware approximation refined by one
 // Newton step.  d is twice a triangle's area, far above the subnormal range
 // for any triangle with vertices on the grid of 2^-24.
@@ -782,7 +811,7 @@ struct NodeCounters {
 template <bool kDebug, bool kCount, bool kExt, bool kCompact>
 __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, NodeCounters &c)
 {
-    const FastProb &P = a.probs[pi];
+    const FastProb &P = a.single ? a.prob0 : a.probs[pi];
     const float4 xq = a.xyq[i];
     const df x = df_make(xq.x, xq.z), y = df_make(xq.y, xq.w);
     df DX, DY;
@@ -807,7 +836,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
         if (kExt && a.exclude && (df_neg_strict(X) || df_gt1(X) || df_neg_strict(Y) || df_gt1(Y))) {
             // the paper's experiments exclude nodes whose foot leaves the
             // domain (Sec. 4): V unchanged, no walk, T^0 unchanged
-            ((float2 *)a.vout)[i] = ((const float2 *)a.vin)[i];
+            keep_value(a, i);
             c.excluded = 1;
             if (a.parent) {
                 // strategy (c): the children start where this node would have
@@ -848,7 +877,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     // rounding-sized offset every step.
     if (at_node && (tq.y == (int32_t)i || tq.z == (int32_t)i || tq.w == (int32_t)i)) {
         const int32_t j0 = tri_of(tq.x);
-        ((float2 *)a.vout)[i] = ((const float2 *)a.vin)[i];
+        keep_value(a, i);
         if (kExt && a.parent && !a.keep_t0) {
             a.t0[i] = j0;
             a.t0v[i] = tq;
@@ -1039,12 +1068,17 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     // FP64 where V^n is steep (SL_OPT_PRECISE)
     {
         const float2 *vin = (const float2 *)a.vin;
-        const float2 V1 = vin[w0], V2 = vin[w1], V3 = vin[w2];
+        float2 V1 = vin[w0], V2 = vin[w1], V3 = vin[w2];
+        if (a.io & kIoIn) {
+            pair_in(a, V1);
+            pair_in(a, V2);
+            pair_in(a, V3);
+        }
         if (!(flags & SL_NODE_CLIPPED) && steep(V1, V2, V3, den.h, a.steep_g2)) {
-            ((float2 *)a.vout)[i] = precise_value(a.xyd, a.g1, a.g2, P, i, w0, w1, w2, V1, V2, V3);
+            put_value(a, i, precise_value(a.xyd, a.g1, a.g2, P, i, w0, w1, w2, V1, V2, V3));
             flags |= SL_NODE_PRECISE;
         } else {
-            ((float2 *)a.vout)[i] = p1_value_of(V1, V2, V3, n1, n2, den);
+            put_value(a, i, p1_value_of(V1, V2, V3, n1, n2, den));
         }
     }
     if ((hops > 0 || (kExt && a.parent)) && !(kExt && a.keep_t0)) {
@@ -1065,7 +1099,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
 // strategies (a), (c) and the direct structured-grid start); the default
 // variant compiles them out and keeps its registers for the walk.
 template <bool kStats, bool kDebug, int kBlock, int kMinBlocks, bool kExt, bool kCompact>
-__global__ void __launch_bounds__(kBlock, kMinBlocks) k_step_fast_df(FastArgs a)
+__global__ void __launch_bounds__(kBlock, kMinBlocks) k_step_fast_df(const __grid_constant__ FastArgs a)
 {
     const int64_t i = kExt ? node_of_thread(a) : (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = kExt ? i >= 0 : i < a.N;
@@ -1139,7 +1173,7 @@ __device__ __forceinline__ int settle_decide(const FastArgs &a, int64_t i, int4 
 template <bool kDebug, int kKind>
 __device__ __forceinline__ bool settle_node(const FastArgs &a, int64_t i, int pi, NodeCounters &c)
 {
-    const FastProb &P = kKind < 0 ? a.probs[pi] : a.prob0;
+    const FastProb &P = kKind >= 0 || a.single ? a.prob0 : a.probs[pi];
     df X, Y;
     bool at_node, gone;
     const bool clipped = foot_pair<kKind>(a, i, P, X, Y, at_node, gone);
@@ -1189,7 +1223,7 @@ __device__ __forceinline__ bool settle_node(const FastArgs &a, int64_t i, int pi
 // kKind >= 0: a single problem of that field kind, whose constants come
 // from the kernel parameters (a.prob0); -1: any problems.
 template <bool kStats, bool kDebug, int kBlock, int kMinBlocks, int kKind>
-__global__ void __launch_bounds__(kBlock, kMinBlocks) k_settle_df(FastArgs a)
+__global__ void __launch_bounds__(kBlock, kMinBlocks) k_settle_df(const __grid_constant__ FastArgs a)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = i < a.N;
@@ -1216,7 +1250,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_settle_df(FastArgs a)
 // Finish pass: the full node step (certified walk, exact stage, value) for
 // the queued nodes, a persistent grid striding over the queue.
 template <bool kStats, bool kDebug, bool kCompact>
-__global__ void __launch_bounds__(128, 8) k_finish_df(FastArgs a)
+__global__ void __launch_bounds__(128, 8) k_finish_df(const __grid_constant__ FastArgs a)
 {
     pdl_launch_dependents();
     pdl_wait();

@@ -116,14 +116,14 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
     const bool clipped = foot_pair<-1, kExt, true>(a, i, P, X, Y, at_node, gone);
     const float2 *vin = (const float2 *)a.vin;
     if (kExt && gone) {
-        ((float2 *)a.vout)[i] = vin[i];
+        keep_value(a, i);
         return true;
     }
     int4 tq = kExt && a.grid_M > 0 ? __ldg(&a.grid_t0v[grid_slot(X.h, Y.h, a.grid_M)]) : a.t0v[i];
     if (at_node) {
         // the foot is its own node: see step_node
         if (tq.y != (int32_t)i && tq.z != (int32_t)i && tq.w != (int32_t)i) return false;
-        ((float2 *)a.vout)[i] = vin[i];
+        keep_value(a, i);
         return true;
     }
     float4 A = a.xyq[tq.y], B = a.xyq[tq.z], C = a.xyq[tq.w];
@@ -168,12 +168,17 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
         C = a.xyq[tq.w];
         moved = true;
     }
+    if (a.io & kIoIn) {
+        pair_in(a, V1);
+        pair_in(a, V2);
+        pair_in(a, V3);
+    }
     float2 val;
     if (!clipped && steep(V1, V2, V3, t.den.h, a.steep_g2))
-        val = precise_value(a.xyd, a.g1, a.g2, a.probs[pi], i, tq.y, tq.z, tq.w, V1, V2, V3);
+        val = precise_value(a.xyd, a.g1, a.g2, P, i, tq.y, tq.z, tq.w, V1, V2, V3);
     else
         val = p1_value_of(V1, V2, V3, t.n1, t.n2, t.den);
-    ((float2 *)a.vout)[i] = val;
+    put_value(a, i, val);
     if (moved && !(kExt && a.keep_t0)) {
         a.t0[i] = tri_of(tq.x);
         a.t0v[i] = tq;

@@ -119,3 +119,64 @@ def test_jump_table_of_uneven_batch():
         finally:
             sl.sl_mesh_destroy(h)
     assert bool((got[0][0] == got[1][0]).all()) and bool((got[0][1] == got[1][1]).all())
+
+
+@pytest.mark.parametrize("split", [0, 1])
+@pytest.mark.parametrize("steps", [1, 2, 3, 4])
+def test_first_and_last_steps_on_doubles(steps, split):
+    """sl_run's first step reads doubles and its last one writes them, on the
+    buffers the number of steps leaves to each; so do single steps.  Values of
+    every magnitude come out as the (hi, lo) pairs of the steps between."""
+    m = si.grid_mesh(70, 0.25, 8)
+    f = si.fourier8_field(3)
+    g = DeviceRun(m, f, 0.02, curve=sl.SL_CURVE_HILBERT)
+    t = g.torch
+    rng = np.random.default_rng(steps)
+    v0 = g.to_dev(rng.standard_normal(m.n_nodes) * np.exp2(rng.integers(-90, 90, m.n_nodes)))
+    v0[:4] = t.tensor([0.0, -0.0, 1e-300, -1e300], dtype=t.float64)
+    # every step through the value conversions: single split steps
+    sl.sl_mesh_set_option(g.h, sl.SL_OPT_SPLIT, 1)
+    start = t.empty(m.n_nodes, dtype=t.int32, device=g.dev)
+    sl.sl_mesh_get_t0(g.h, start)
+    for initial in (True, False):
+        ref, w = v0.clone(), t.empty_like(v0)
+        sl.sl_mesh_set_t0(g.h, start)          # no longer "initial": split from the first step
+        for n in range(steps):
+            sl.sl_step(g.h, g.probs, n, ref, w)
+            ref, w = w, ref
+        sl.sl_mesh_set_option(g.h, sl.SL_OPT_SPLIT, split)
+        (sl.sl_mesh_reset_t0(g.h) if initial else sl.sl_mesh_set_t0(g.h, start))
+        v, w = v0.clone(), t.empty_like(v0)
+        sl.sl_run(g.h, g.probs, 0, steps, v, w)
+        assert np.array_equal(v.cpu().numpy().view(np.int64), ref.cpu().numpy().view(np.int64))
+        (sl.sl_mesh_reset_t0(g.h) if initial else sl.sl_mesh_set_t0(g.h, start))
+        v, w = v0.clone(), t.empty_like(v0)
+        for n in range(steps):
+            sl.sl_step(g.h, g.probs, n, v, w)
+            v, w = w, v
+        assert np.array_equal(v.cpu().numpy().view(np.int64), ref.cpu().numpy().view(np.int64))
+        sl.sl_mesh_set_option(g.h, sl.SL_OPT_SPLIT, 1)
+
+
+def test_single_steps_of_a_batch_follow_their_constants():
+    """A batch of more problems than one launch of constants takes, stepped
+    without a synchronisation in between."""
+    import torch
+    meshes = [si.grid_mesh(3 + k % 9, 0.25, k) for k in range(70)]
+    fields = [si.rotation_field(1.0 + 0.1 * k) for k in range(70)]
+    no, to, xy, tri = sl.pack_meshes([(m.xy, m.tri) for m in meshes])
+    probs = sl.problems([(f.kind, 0.05, f.packed()) for f in fields])
+    v0 = torch.tensor(np.concatenate([si.gaussian(m.xy) for m in meshes]), dtype=torch.float64, device="cuda")
+    h = sl.sl_mesh_create(no, to, xy, tri)
+    try:
+        v, w = v0.clone(), torch.empty_like(v0)
+        sl.sl_run(h, probs, 0, 5, v, w)
+        sl.sl_mesh_reset_t0(h)
+        a, b = v0.clone(), torch.empty_like(v0)
+        for n in range(5):
+            sl.sl_step(h, probs, n, a, b)
+            a, b = b, a
+        # pairs between the steps of a run, doubles between single steps: 48 bits
+        assert float((a - v).abs().max()) <= 5 * 2.0 ** -46
+    finally:
+        sl.sl_mesh_destroy(h)
