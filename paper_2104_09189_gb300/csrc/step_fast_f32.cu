@@ -100,7 +100,8 @@ struct CountersF32 {
 // kExt: the variant with the options of the paper's experiments (exclusion,
 // strategies (a), (c) and the direct structured-grid start); the default
 // variant compiles them out.
-template <bool kDebug, bool kExt>
+// kCount: the variants that count or report (statistics, debug outputs).
+template <bool kDebug, bool kCount, bool kExt>
 __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int pi, CountersF32 &c)
 {
     const FastProb &P = a.single ? a.prob0 : a.probs[pi];
@@ -219,6 +220,18 @@ __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int 
                 float xb = X, yb = Y;
                 asm volatile("" : "+f"(xb), "+f"(yb));
                 const double Xd = xb, Yd = yb;
+                if (!kCount) {
+                    // integers where the coordinates allow (the counting variants
+                    // take the stages below, which give the same signs)
+                    long long ax, ay, bx, by, cx, cy, x, y;
+                    if (slp::fixed62(A.x, ax) & slp::fixed62(A.y, ay) & slp::fixed62(B.x, bx) &
+                        slp::fixed62(B.y, by) & slp::fixed62(C.x, cx) & slp::fixed62(C.y, cy) & slp::fixed62(Xd, x) &
+                        slp::fixed62(Yd, y)) {
+                        if (s1 == 2) s1 = slp::orient_fixed62(bx, by, cx, cy, x, y);
+                        if (s2 == 2) s2 = slp::orient_fixed62(cx, cy, ax, ay, x, y);
+                        if (s3 == 2) s3 = slp::orient_fixed62(ax, ay, bx, by, x, y);
+                    }
+                }
                 if (s1 == 2) {
                     slp::OrientResult r = slp::orient(B.x, B.y, C.x, C.y, Xd, Yd);
                     s1 = r.sign;
@@ -380,7 +393,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_step_fast_f32(const __gr
                    : (kExt && a.order ? problem_of(a.node_off, a.nprob, i) : chunk_problem(a.chunk_prob, a.node_off, i));
     pdl_launch_dependents();
     pdl_wait();
-    if (active) step_node_f32<kDebug, kExt>(a, i, pi, c);
+    if (active) step_node_f32<kDebug, kStats || kDebug, kExt>(a, i, pi, c);
     if (kStats)
         warp_stats(a.stats, active, c.hops, c.exact_tests, c.clipped_cnt, c.fallback_cnt, c.limit_cnt, c.fp64_tests,
                    c.excluded_cnt);
@@ -550,7 +563,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_lean_f32(const __grid_co
     const int pi = kSingle || a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i);
     if (lean_node_f32<kExt, kSingle>(a, i, pi)) return;
     CountersF32 c;
-    step_node_f32<false, kExt>(a, i, pi, c);
+    step_node_f32<false, false, kExt>(a, i, pi, c);
 }
 
 template <int kBlock, int kMinBlocks, bool kExt = false>

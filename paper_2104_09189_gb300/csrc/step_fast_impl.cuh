@@ -247,6 +247,9 @@ __device__ __forceinline__ float cert_bound_g(float S) { return S * __fmaf_rn(S,
 // Packed result: bits 2k..2k+1 the sign of edge k (0: 0, 1: +1, 2: -1),
 // bits 8..9 the tests decided by the expansion, bits 10..11 those decided by
 // the double filter, bit 12 a coordinate outside the exact range.
+// kCount: the stages are counted; otherwise integers decide where they can
+// (slp::fixed62), with the same signs.
+template <bool kCount>
 __device__ __forceinline__ uint32_t exact_signs(const double2 *xyd, int w0, int w1, int w2, df X, df Y, uint32_t need)
 {
     // The foot is loop-invariant: without this barrier the compiler hoists
@@ -255,6 +258,20 @@ __device__ __forceinline__ uint32_t exact_signs(const double2 *xyd, int w0, int 
     asm volatile("" : "+f"(X.h), "+f"(X.l), "+f"(Y.h), "+f"(Y.l));
     const double2 Ad = xyd[w0], Bd = xyd[w1], Cd = xyd[w2];
     uint32_t out = 0, n3 = 0, n2 = 0;
+    if (!kCount) {
+        long long ax, ay, bx, by, cx, cy, xh, xl, yh, yl;
+        bool ok = slp::fixed62(Ad.x, ax) & slp::fixed62(Ad.y, ay) & slp::fixed62(Bd.x, bx) & slp::fixed62(Bd.y, by) &
+                  slp::fixed62(Cd.x, cx) & slp::fixed62(Cd.y, cy) & slp::fixed62(X.h, xh) & slp::fixed62(X.l, xl) &
+                  slp::fixed62(Y.h, yh) & slp::fixed62(Y.l, yl);
+        const long long x = xh + xl, y = yh + yl;
+        ok = ok && x >= 0 && x <= 1ll << 62 && y >= 0 && y <= 1ll << 62;
+        if (ok) {
+            const int s0 = slp::orient_fixed62(bx, by, cx, cy, x, y), s1 = slp::orient_fixed62(cx, cy, ax, ay, x, y),
+                      s2 = slp::orient_fixed62(ax, ay, bx, by, x, y);
+            return (s0 > 0 ? 1u : (s0 < 0 ? 2u : 0u)) | (s1 > 0 ? 4u : (s1 < 0 ? 8u : 0u)) |
+                   (s2 > 0 ? 16u : (s2 < 0 ? 32u : 0u));
+        }
+    }
     for (int k = 0; k < 3; ++k) {
         if (!(need >> k & 1u)) continue;
         const double2 P = k == 0 ? Bd : (k == 1 ? Cd : Ad), Q = k == 0 ? Cd : (k == 1 ? Ad : Bd);
@@ -999,7 +1016,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
                 need &= r >> 8;
             }
             // exact signs on the double coordinates and the exact foot
-            const uint32_t r = need ? exact_signs(a.xyd, w0, w1, w2, X, Y, need) : 0u;
+            const uint32_t r = need ? exact_signs<kCount>(a.xyd, w0, w1, w2, X, Y, need) : 0u;
             if (s1 == 2) s1 = unpack_sign(r, 0);
             if (s2 == 2) s2 = unpack_sign(r, 1);
             if (s3 == 2) s3 = unpack_sign(r, 2);

@@ -97,6 +97,27 @@ def test_feet_on_edges_and_vertices(precision):
             v = b
 
 
+@pytest.mark.parametrize("precision", [sl.SL_FP64, sl.SL_FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -8, 2.0 ** -40], ids=["unit", "2^-8", "2^-40"])
+def test_exact_signs_near_a_corner(scale, precision):
+    """Feet on the lines of a grid whose first cells are `scale` / 16 wide: decided
+    in integers where the coordinates are multiples of 2^-62, by the expansions
+    where they are not."""
+    c = np.concatenate([np.arange(16) / 16.0 * scale, [1.0] if scale == 1.0 else [scale, 0.5, 1.0]])
+    n = len(c)
+    xy = np.stack(np.meshgrid(c, c, indexing="xy"), -1).reshape(-1, 2)
+    a = (np.arange(n - 1)[:, None] * n + np.arange(n - 1)[None, :]).ravel()
+    tri = np.stack([a, a + n + 1, a + n, a, a + 1, a + n + 1], 1).reshape(-1, 3).astype(np.int32)
+    m = si.Mesh(M=n - 1, xy=xy, tri=tri)
+    f = si.affine_field([3.5 / 16 * scale, 0, 0, 0, 2.0 / 16 * scale, 0, 0, 0])
+    g = DeviceRun(m, f, 1.0, precision=precision)
+    v = g.to_dev(np.sin(np.arange(n * n)))
+    for k in range(2):
+        (p, q), (jp, jq) = step_both(g, k, v)
+        assert bool((jp == jq).all()) and bool((p == q).all()), f"step {k}"
+        v = q
+
+
 def test_jump_table_of_uneven_batch():
     """Meshes of 9 to 10 000 nodes in one batch, each with a table of its own."""
     import torch
