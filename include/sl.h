@@ -135,7 +135,7 @@ typedef enum {
     SL_OPT_BLOCK = 3,        /* threads per block of the plain FP64 kernel (0 = auto) */
     /* 4 and 6 are not options (SL_E_ARG) */
     SL_OPT_CONFIG = 5,       /* launch configuration of the fast kernels, 0..5: threads per block x
-                                blocks per SM the registers are sized for = 256x4, 256x3, 128x8,
+                                blocks per SM the registers are sized for = 256x4, 128x16, 128x8,
                                 128x9, 256x5, 128x12 (default 5) */
     SL_OPT_CONFIG_FIRST = 7, /* launch configuration for a step whose walks start at the initial
                                 incident triangles (the first step after sl_mesh_create or

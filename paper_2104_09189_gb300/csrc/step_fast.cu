@@ -74,8 +74,9 @@ void launch_finish_df(const FastArgs &a, bool stats, bool debug, int sms, cudaSt
 
 
 // Launch configurations (threads per block x resident blocks per SM the
-// register budget is sized for): 0 = 256 x 4 (64 registers), 1 = 256 x 3,
-// 2 = 128 x 8, 3 = 128 x 9 (56 registers), 4 = 256 x 5, 5 = 128 x 12.  Each
+// register budget is sized for): 0 = 256 x 4 (64 registers), 1 = 128 x 16 (32;
+// 2 % faster than 128 x 12 on a batch of 2.8 M nodes, 4 % slower on 491 k), 2 =
+// 128 x 8, 3 = 128 x 9 (56 registers), 4 = 256 x 5, 5 = 128 x 12.  Each
 // is instantiated in a translation unit of its own pair (step_fast_c*.cu).
 //
 // They are configurations of the lean kernel.  Statistics, debug outputs and

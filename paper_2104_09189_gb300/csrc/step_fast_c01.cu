@@ -7,6 +7,6 @@ namespace sl {
 
 void launch_lean_df_c0(const FastArgs &a, cudaStream_t s) { launch_lean_df_cfg<256, 4>(a, s); }
 
-void launch_lean_df_c1(const FastArgs &a, cudaStream_t s) { launch_lean_df_cfg<256, 3>(a, s); }
+void launch_lean_df_c1(const FastArgs &a, cudaStream_t s) { launch_lean_df_cfg<128, 16>(a, s); }
 
 }  // namespace sl
