@@ -277,10 +277,11 @@ sl_status sl_step(sl_mesh *m, const sl_problem *probs, int64_t n, const void *v_
 /*
  * sl_run -- n_steps steps from n0 (Algorithm 2's time loop).  `v` (device,
  * N values) holds V^{n0} on entry and V^{n0+n_steps} on return; `v_scratch`
- * (device, N values) is used for the ping-pong.  With use_graph != 0 the
- * steps are recorded once into a CUDA graph and replayed (the graph is kept
- * in the handle and reused while n0, n_steps, the buffers and the problems
- * are unchanged).  Synchronises the stream and returns the deferred device
+ * (device, N values) is used for the ping-pong.  With use_graph != 0 a run
+ * that repeats the one before (the same n0, n_steps, buffers and problems) is
+ * recorded into a CUDA graph, which is kept in the handle and replayed while
+ * they are unchanged; the first run with new arguments is launched step by
+ * step.  Synchronises the stream and returns the deferred device
  * status (SL_E_WALK_LIMIT if a walk failed).  stats may be NULL; with
  * SL_OPT_ASYNC = 1 and stats NULL it returns without synchronising.
  */

@@ -159,15 +159,21 @@ def _ptr(x):
     raise TypeError(f"cannot take the address of {type(x)}")
 
 
+_torch = None      # the torch module once a CUDA device has been seen
+
+
 def _stream(stream):
+    global _torch
     if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream
-        except ImportError:
-            pass
-        return None
+        if _torch is None:
+            try:
+                import torch
+                if not torch.cuda.is_available():
+                    return None
+                _torch = torch
+            except ImportError:
+                return None
+        return _torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -60,8 +60,8 @@ struct DeviceMesh {
 };
 
 struct GraphCache {
-    bool valid = false;
-    void *exec = nullptr;             // cudaGraphExec_t
+    bool valid = false;               // the fields below describe the last run with use_graph
+    void *exec = nullptr;             // cudaGraphExec_t of that run, or NULL: launched, not recorded
     int64_t n0 = 0;
     int32_t n_steps = 0;
     const void *v = nullptr, *v_scratch = nullptr;
@@ -119,6 +119,7 @@ struct sl_mesh {
     sl::GraphCache graph;
     // device value buffers for sl_run_host
     void *host_v = nullptr, *host_v2 = nullptr;
+    void *report = nullptr;           // page-locked: status words and counters as read back
     void *capture_stream = nullptr;   // cudaStream_t used only to record graphs
 };
 
