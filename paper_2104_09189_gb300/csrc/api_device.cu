@@ -114,7 +114,7 @@ void free_device(sl_mesh *m)
     release_l2_window(m);
     DeviceMesh &d = m->d;
     void *ptrs[] = {d.xy, d.tv[0], d.tv[1], d.tv[2], d.tn[0], d.tn[1], d.tn[2], d.t0, d.t0_init, d.t0v, d.node_off, d.chunk_prob,
-                    d.status, d.probs, d.fprobs, d.xyq, d.xyh, d.g1, d.g2, d.tparams, d.dfa, d.dfb, d.he, d.he8, d.tri, d.jump, d.grid_t0v, d.tree_order, d.tree_parent, d.queue, d.queue_count,
+                    d.status, d.probs, d.fprobs, d.xyq, d.xyh, d.g1, d.g2, d.tparams, d.dfa, d.dfb, d.he, d.he8, d.wq, d.wt, d.tri, d.jump, d.grid_t0v, d.tree_order, d.tree_parent, d.queue, d.queue_count,
                     m->host_v, m->host_v2};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -447,6 +447,9 @@ FastArgs make_fast_args(const sl_mesh *m, const FastProb *fp, const void *vin, v
     // walk itself
     a.jump = m->opt_strategy == 0 && m->opt_walk_cap == 0 ? (const int4 *)m->d.jump : nullptr;
     a.t0_init = m->d.t0_init;
+    a.wq = (int4 *)m->d.wq;
+    if (m->precision == SL_FP64) a.wt = (float4 *)m->d.wt;
+    else a.wt2 = (float *)m->d.wt;
     a.t0 = m->d.t0;
     a.t0v = (int4 *)m->d.t0v;
     a.vin = vin;
@@ -671,6 +674,23 @@ static sl_status launch_fast(sl_mesh *m, const FastArgs &a, bool debug, int conf
     return SL_OK;
 }
 
+// Step k of a run of steady fields: the first one in the fused kernel (which
+// stores the weights), the others apply them.
+static sl_status launch_steady(sl_mesh *m, const FastArgs &a, int config, int32_t k, cudaStream_t s)
+{
+    FastArgs x = a;
+    x.pdl = m->opt_pdl && k > 0;
+    if (m->precision == SL_FP64) {
+        if (k == 0) launch_fast_df(x, false, false, config, s);
+        else launch_apply_df(x, s);
+    } else {
+        if (k == 0) launch_fast_f32(x, false, false, config, s);
+        else launch_apply_f32(x, s);
+    }
+    SL_CUDA(cudaGetLastError());
+    return SL_OK;
+}
+
 static sl_status check_device(const sl_mesh *m)
 {
     int dev = -1;
@@ -722,6 +742,40 @@ static sl_status ensure_fprobs(sl_mesh *m, size_t bytes)
     SL_CUDA(cudaMalloc(&m->d.fprobs, bytes));
     m->d.fprobs_bytes = bytes;
     return SL_OK;
+}
+
+// Steady fields of a run (emit_weights): problems whose constants are the same
+// at every one of the n_steps steps store their weights at the first step and
+// use them at the others.  Marks them in fh and returns whether all of them
+// are.  Storing costs about half a later step's time once and saves a third of
+// one per step, so runs of fewer than 4 steps go without; so do the counting
+// variants, the paper's experiments, split steps of a batch that is only
+// partly steady, and a device without room for the weights.
+constexpr int32_t kSteadySteps = 4;
+static bool mark_steady(sl_mesh *m, int32_t n_steps, bool split_rest, std::vector<FastProb> &fh)
+{
+    if (n_steps < kSteadySteps || m->opt_stats || m->opt_strategy != 0 || m->opt_outside) return false;
+    const int32_t np = m->n_problems;
+    std::vector<uint8_t> steady(np, 1);
+    bool any = false, all = true;
+    for (int32_t p = 0; p < np; ++p) {
+        for (int32_t k = 1; k < n_steps && steady[p]; ++k)
+            steady[p] = std::memcmp(&fh[(size_t)k * np + p], &fh[p], sizeof(FastProb)) == 0;
+        any |= steady[p] != 0;
+        all &= steady[p] != 0;
+    }
+    if (!any || (split_rest && !all)) return false;
+    if (!m->d.wq || !m->d.wt) {
+        const size_t tsz = m->precision == SL_FP64 ? sizeof(float4) : sizeof(float);
+        if ((!m->d.wq && cudaMalloc(&m->d.wq, sizeof(int4) * m->N) != cudaSuccess) ||
+            (!m->d.wt && cudaMalloc(&m->d.wt, tsz * m->N) != cudaSuccess)) {
+            cudaGetLastError();     // no room: the steps locate every time
+            return false;
+        }
+    }
+    for (int32_t p = 0; p < np; ++p)
+        for (int32_t k = 0; k < n_steps && steady[p]; ++k) fh[(size_t)k * np + p].flags |= k == 0 ? kFastEmit : kFastUse;
+    return all;
 }
 
 static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int32_t n_steps, void *v, void *v2,
@@ -784,11 +838,13 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
     };
     auto config_of = [&](int32_t k) { return (k == 0 && first_initial) ? m->opt_config_first : m->opt_config; };
     std::vector<FastProb> fh;   // the fast kernels' constants, host copy (filled when recording)
+    bool all_steady = false;
     if (!reuse) {
         if (fast) {
             fh.resize((size_t)m->n_problems * (size_t)n_steps);
             for (int32_t k = 0; k < n_steps; ++k)
                 fill_fast(m, host.data() + (size_t)k * m->n_problems, fh.data() + (size_t)k * m->n_problems);
+            all_steady = mark_steady(m, n_steps, split_step(m, false), fh);
             if (m->n_problems > 1) {
                 // (a single problem's constants are kernel parameters.)  A
                 // synchronous copy: a graph recorded below may replay them later
@@ -810,7 +866,8 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
             // first step reads the doubles itself and a last one writes them
             // where the number of steps puts them on the right buffers (the
             // passes of a split step take pairs only)
-            const bool can_in = !split_step(m, first_initial), can_out = !split_step(m, n_steps == 1 && first_initial);
+            const bool can_in = !split_step(m, first_initial) || all_steady,
+                       can_out = !split_step(m, n_steps == 1 && first_initial) || all_steady;
             const bool in = can_in && (n_steps % 2 == 0 || !can_out), out = can_out && in == (n_steps % 2 == 0);
             void *a = v, *b = v2;
             if (!in) {
@@ -823,7 +880,9 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
                 FastArgs args = make_fast_args(m, (const FastProb *)((char *)m->d.fprobs + fper * k), a, b, nullptr,
                                                fh.data() + (size_t)k * m->n_problems);
                 args.io = (in && k == 0 ? kIoIn : 0) | (out && k == n_steps - 1 ? kIoOut : 0);
-                sl_status st = launch_fast(m, args, false, config_of(k), k == 0 && first_initial, q, &split_seq, k > 0);
+                sl_status st = all_steady ? launch_steady(m, args, config_of(k), k, q)
+                                          : launch_fast(m, args, false, config_of(k), k == 0 && first_initial, q,
+                                                        &split_seq, k > 0);
                 if (st != SL_OK) return st;
                 void *t = a;
                 a = b;
@@ -840,7 +899,9 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
             if (fast) {
                 FastArgs args = make_fast_args(m, (const FastProb *)((char *)m->d.fprobs + fper * k), a, b, nullptr,
                                                fh.data() + (size_t)k * m->n_problems);
-                st = launch_fast(m, args, false, config_of(k), k == 0 && first_initial, q, &split_seq, k > 0);
+                st = all_steady ? launch_steady(m, args, config_of(k), k, q)
+                                : launch_fast(m, args, false, config_of(k), k == 0 && first_initial, q, &split_seq,
+                                              k > 0);
             } else {
                 StepArgs args = make_args(m, (const ProbStep *)((char *)m->d.probs + per * k), a, b, nullptr);
                 st = launch_step(m, args, false, q);

@@ -54,6 +54,7 @@ struct DeviceMesh {
     double *tparams = nullptr;        // field parameters the tables were built from (device)
     void *dfa = nullptr, *dfb = nullptr;   // value scratch of sl_step for the fast FP64 kernel
     void *he = nullptr;               // float4 half-edge walk records of the fast kernels (3 Nt), or NULL
+    void *wq = nullptr, *wt = nullptr;   // a run's steady weights per node (FastArgs; FP32: wt holds wt2)
     void *tri = nullptr;              // int4 (3 t, its vertex ids) per triangle
     void *jump = nullptr;             // int4 start state per cell of the problems' jump tables
     void *he8 = nullptr;              // uint2 compact records (FP64 meshes that fit, 3 Nt), or NULL

@@ -101,6 +101,27 @@ void launch_fast_df(const FastArgs &a, bool stats, bool debug, int config, cudaS
     }
 }
 
+// A later step of steady fields (apply_weights) for every node.  Bound by
+// memory: 48 bytes per node stream (weights, V^n, V^{n+1}) beside three value
+// gathers that mostly hit L1, at 32 registers and 64 warps per SM: 0.118 ms on
+// 16.8 M nodes, the measured copy bandwidth, where locating every node again
+// (foot, certified test, quotient; also 48 bytes, 290 instructions, 64 bytes of
+// gathered vertices) took 0.180 ms.  A 50-step rotation 9.60 -> 6.69 ms.  The
+// weights past L1: they are read once.
+__global__ void __launch_bounds__(256, 8) k_apply_df(const __grid_constant__ FastArgs a)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (i < a.N) put_value(a, i, apply_weights(a, i));
+}
+
+void launch_apply_df(const FastArgs &a, cudaStream_t s)
+{
+    const unsigned grid = (unsigned)((a.N + 255) / 256);
+    if (grid) launch_step_kernel(k_apply_df, grid, 256, s, a);
+}
+
 // ---------------------------------------------------------------------------
 // Gather probe: the memory accesses of a step whose feet stay in their start
 // triangles, with only a sum as arithmetic (sl_probe_gather).

@@ -25,7 +25,7 @@ namespace sl {
 // in float, and x - c costs two additions.
 struct FastProb {
     int32_t kind;
-    int32_t flags;      // kFastCentreGrid
+    int32_t flags;      // kFastCentreGrid, kFastEmit, kFastUse
     int32_t jump_g;     // cells per side of the problem's jump table
     int32_t jump_off;   // its first cell in FastArgs::jump
     float2 c[6];        // (hi, lo)
@@ -33,6 +33,11 @@ struct FastProb {
 
 constexpr int32_t kFastCentreGrid = 1;
 constexpr int32_t kIoIn = 1, kIoOut = 2;
+// FastProb::flags of a run's steps for a problem whose constants are the same
+// at every step: its feet, triangles and barycentric coordinates are too.  The
+// first step stores them (kFastEmit), the others interpolate with them
+// (kFastUse); see emit_weights.
+constexpr int32_t kFastEmit = 2, kFastUse = 4;
 
 // The six per-step constants of a problem as float pairs: (hi, lo), or for a
 // rotation centre in [0, 1]^2 the (grid, remainder) split of the node
@@ -63,6 +68,10 @@ struct FastArgs {
                                   // passes of a split step.
     const float4 *g1, *g2;        // field tables (hi, lo) per node (FP64 meshes), or NULL
     const float2 *g1f, *g2f;      // field tables rounded to float (FP32 meshes), or NULL
+    // a node's triangle and barycentric coordinates within one run (emit_weights)
+    int4 *wq;                     // FP64: vertex ids, steepness threshold; FP32: vertex ids, theta_1
+    float4 *wt;                   // FP64: theta_1, theta_2 as (hi, lo) pairs
+    float *wt2;                   // FP32: theta_2
     const FastProb *probs;
     FastProb prob0;               // single: a copy of probs[0] (kernel parameter space)
     int32_t single;               // one problem, prob0 valid
@@ -183,6 +192,10 @@ void launch_settle_df(const FastArgs &a, bool stats, bool debug, bool reset, cud
 void launch_finish_df(const FastArgs &a, bool stats, bool debug, int sms, cudaStream_t s);
 constexpr int kFastConfigs = 6;
 void launch_fast_f32(const FastArgs &a, bool stats, bool debug, int config, cudaStream_t s);
+
+// a step of problems that all have kFastUse
+void launch_apply_df(const FastArgs &a, cudaStream_t s);
+void launch_apply_f32(const FastArgs &a, cudaStream_t s);
 
 // the memory accesses of a steady step with no arithmetic (sl_probe_gather)
 void launch_gather_probe(const float4 *xyq, const int4 *t0v, const float2 *vin, float2 *vout, int64_t N,

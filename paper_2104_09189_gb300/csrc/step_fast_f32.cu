@@ -91,6 +91,46 @@ __device__ __forceinline__ int32_t tri_of_f32(int32_t h) { return (int32_t)__umu
 // orientation was certified negative from the other side, so here it is
 // positive.  The value is evaluated with the located triangle's vertices in
 // slot order, so it does not depend on the path of the walk.
+// Steady fields within a run, as emit_weights and apply_weights of the
+// double-float kernel: the vertex ids and theta_1 in 16 bytes, theta_2 in 4.  The
+// later steps' values are the same bits.
+__device__ __forceinline__ float interpolate_f32(float th1, float th2, float v1, float v2, float v3)
+{
+    return __fmaf_rn(th1, __fsub_rn(v1, v3), __fmaf_rn(th2, __fsub_rn(v2, v3), v3));
+}
+
+__device__ __forceinline__ void emit_weights_f32(const FastArgs &a, int64_t i, int w0, int w1, int w2, float th1,
+                                                 float th2)
+{
+    a.wq[i] = make_int4(w0, w1, w2, __float_as_int(th1));
+    a.wt2[i] = th2;
+}
+
+__device__ __forceinline__ void apply_weights_f32(const FastArgs &a, int64_t i)
+{
+    int4 w;
+    asm volatile("ld.global.L1::no_allocate.v4.s32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(a.wq + i));
+    const float th2 = a.wt2[i];
+    const float *vin = (const float *)a.vin;
+    const float v1 = vin[w.x], v2 = vin[w.y], v3 = vin[w.z];
+    ((float *)a.vout)[i] = interpolate_f32(__int_as_float(w.w), th2, v1, v2, v3);
+}
+
+__global__ void __launch_bounds__(256, 8) k_apply_f32(const __grid_constant__ FastArgs a)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    if (i < a.N) apply_weights_f32(a, i);
+}
+
+void launch_apply_f32(const FastArgs &a, cudaStream_t s)
+{
+    const unsigned grid = (unsigned)((a.N + 255) / 256);
+    if (grid) launch_step_kernel(k_apply_f32, grid, 256, s, a);
+}
+
 struct CountersF32 {
     uint32_t hops = 0, exact_tests = 0, clipped_cnt = 0, fallback_cnt = 0, limit_cnt = 0, fp64_tests = 0;
     uint32_t excluded_cnt = 0;
@@ -357,8 +397,8 @@ __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int 
         const float th1 = __fmul_rn(o1, r), th2 = __fmul_rn(o2, r);
         const float *vin = (const float *)a.vin;
         const float v1 = vin[w0], v2 = vin[w1], v3 = vin[w2];
-        const float v = __fmaf_rn(th1, __fsub_rn(v1, v3), __fmaf_rn(th2, __fsub_rn(v2, v3), v3));
-        ((float *)a.vout)[i] = v;
+        ((float *)a.vout)[i] = interpolate_f32(th1, th2, v1, v2, v3);
+        if (!kCount && (P.flags & kFastEmit)) emit_weights_f32(a, i, w0, w1, w2, th1, th2);
         if ((moved || (kExt && a.parent)) && !(kExt && a.keep_t0)) {
             a.t0[i] = j;
             a.t0v[i] = make_int4(3 * j, w0, w1, w2);
@@ -425,6 +465,10 @@ template <bool kExt, bool kSingle>
 __device__ __forceinline__ bool lean_node_f32(const FastArgs &a, int64_t i, int pi)
 {
     const FastProb &P = kSingle ? a.prob0 : a.probs[pi];
+    if (!kSingle && (P.flags & kFastUse)) {
+        apply_weights_f32(a, i);
+        return true;
+    }
     const float *vin = (const float *)a.vin;
     const float2 xf = a.xyf[i];
     float X, Y;
@@ -545,7 +589,8 @@ __device__ __forceinline__ bool lean_node_f32(const FastArgs &a, int64_t i, int 
     const float dn = __fadd_rn(__fadd_rn(o1, o2), o3);
     const float r = __frcp_rn(dn);
     const float th1 = __fmul_rn(o1, r), th2 = __fmul_rn(o2, r);
-    ((float *)a.vout)[i] = __fmaf_rn(th1, __fsub_rn(v1, v3), __fmaf_rn(th2, __fsub_rn(v2, v3), v3));
+    ((float *)a.vout)[i] = interpolate_f32(th1, th2, v1, v2, v3);
+    if (P.flags & kFastEmit) emit_weights_f32(a, i, tq.y, tq.z, tq.w, th1, th2);
     if (moved && !(kExt && a.keep_t0)) {
         a.t0[i] = tri_of_f32(tq.x);
         a.t0v[i] = tq;

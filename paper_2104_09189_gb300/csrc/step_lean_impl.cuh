@@ -111,6 +111,10 @@ template <bool kExt, bool kCompact, bool kSingle>
 __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
 {
     const FastProb &P = kSingle ? a.prob0 : a.probs[pi];
+    if (!kSingle && (P.flags & kFastUse)) {
+        put_value(a, i, apply_weights(a, i));
+        return true;
+    }
     df X, Y;
     bool at_node, gone;
     const bool clipped = foot_pair<-1, kExt, true>(a, i, P, X, Y, at_node, gone);
@@ -124,6 +128,7 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
         // the foot is its own node: see step_node
         if (tq.y != (int32_t)i && tq.z != (int32_t)i && tq.w != (int32_t)i) return false;
         keep_value(a, i);
+        if (P.flags & kFastEmit) emit_own(a, i);
         return true;
     }
     float4 A = a.xyq[tq.y], B = a.xyq[tq.z], C = a.xyq[tq.w];
@@ -179,6 +184,7 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
     else
         val = p1_value_of(V1, V2, V3, t.n1, t.n2, t.den);
     put_value(a, i, val);
+    if (P.flags & kFastEmit) emit_weights(a, i, tq.y, tq.z, tq.w, t.n1, t.n2, t.den, clipped);
     if (moved && !(kExt && a.keep_t0)) {
         a.t0[i] = tri_of(tq.x);
         a.t0v[i] = tq;

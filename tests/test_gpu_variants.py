@@ -201,3 +201,74 @@ def test_single_steps_of_a_batch_follow_their_constants():
         assert float((a - v).abs().max()) <= 5 * 2.0 ** -46
     finally:
         sl.sl_mesh_destroy(h)
+
+
+STEADY = {
+    "rotation": lambda: si.rotation_field(),
+    "zero": lambda: si.zero_field(),
+    "affine": lambda: si.affine_field([0.5, -0.3, 0.2, 0.0, 0.3, 0.1, 0.3, 0.0]),
+}
+
+
+def runs_of(h, probs, v0, chunks):
+    """The values and T0 after runs of the given numbers of steps."""
+    import torch
+    v, w = v0.clone(), torch.empty_like(v0)
+    sl.sl_mesh_reset_t0(h)
+    n = 0
+    for c in chunks:
+        sl.sl_run(h, probs, n, c, v, w)
+        n += c
+    t0 = torch.empty(v.numel(), dtype=torch.int32, device="cuda")
+    sl.sl_mesh_get_t0(h, t0)
+    return v, t0
+
+
+@pytest.mark.parametrize("precise", [0, 1, 32])
+@pytest.mark.parametrize("split", [0, 1])
+@pytest.mark.parametrize("precision", [sl.SL_FP64, sl.SL_FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("field", list(STEADY))
+def test_steady_fields_keep_their_weights(field, precision, split, precise):
+    """Runs of 4 steps and more of a steady field store the weights at the first
+    step; runs of 3 and fewer locate at every step.  (Feet that are their
+    nodes, clipped feet and steep data included.)"""
+    m = si.grid_mesh(75, 0.25, 9)
+    g = DeviceRun(m, STEADY[field](), 0.05, curve=sl.SL_CURVE_HILBERT, precision=precision)
+    sl.sl_mesh_set_option(g.h, sl.SL_OPT_SPLIT, split)
+    sl.sl_mesh_set_option(g.h, sl.SL_OPT_PRECISE, precise)
+    rng = np.random.default_rng(1)
+    v0 = g.to_dev(si.gaussian(m.xy) + 1e-3 * rng.standard_normal(m.n_nodes))
+    a, ta = runs_of(g.h, g.probs, v0, (3, 3, 1))
+    for chunks in ((7,), (4, 3), (2, 5)):
+        b, tb = runs_of(g.h, g.probs, v0, chunks)
+        assert bool((ta == tb).all())
+        if precision == sl.SL_FP32:
+            assert bool((a == b).all())
+        else:
+            # one step: theta_k within 2^-44 and the sums within 2^-46 of |V|, an
+            # interpolation of the errors before it; between runs also the 48
+            # bits of a pair
+            assert float((a - b).abs().max()) <= 7 * 2.0 ** -43 * float(v0.abs().max())
+
+
+@pytest.mark.parametrize("precision", [sl.SL_FP64, sl.SL_FP32], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("kinds", [("rotation", "swirl", "zero", "affine"), ("rotation", "zero", "affine", "rotation")])
+def test_batch_of_steady_and_other_fields(kinds, precision):
+    import torch
+    fields = [STEADY[k]() if k in STEADY else si.swirl_field() for k in kinds]
+    meshes = [si.grid_mesh(M, 0.25, M) for M in (31, 64, 2, 45)]
+    no, to, xy, tri = sl.pack_meshes([(m.xy, m.tri) for m in meshes])
+    probs = sl.problems([(f.kind, 0.04, f.packed()) for f in fields])
+    dt = torch.float64 if precision == sl.SL_FP64 else torch.float32
+    v0 = torch.tensor(np.concatenate([si.gaussian(m.xy) for m in meshes]), dtype=dt, device="cuda")
+    h = sl.sl_mesh_create(no, to, xy, tri, precision=precision)
+    try:
+        a, ta = runs_of(h, probs, v0, (3, 3, 2))
+        for split in (0, 1):
+            sl.sl_mesh_set_option(h, sl.SL_OPT_SPLIT, split)
+            for _ in range(3):      # launched, recorded, replayed
+                b, tb = runs_of(h, probs, v0, (8,))
+                assert bool((ta == tb).all())
+                assert float((a - b).abs().max()) <= (8 * 2.0 ** -43 if precision == sl.SL_FP64 else 0.0)
+    finally:
+        sl.sl_mesh_destroy(h)
