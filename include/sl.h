@@ -323,7 +323,7 @@ sl_status sl_run_host(sl_mesh *m, const sl_problem *probs, int64_t n0, int32_t n
  * on the mesh (that call allocates them); otherwise SL_E_STATE.
  *
  * A batch's per-problem constants live in one library-owned static device
- * array per GPU (16 KiB), held by every GPU that loads the library until the
+ * array per GPU (18 KiB), held by every GPU that loads the library until the
  * process exits; they reach it in the parameters of a small kernel (a single
  * problem's are parameters of the step).  No host buffer of the call is read
  * after it returns.  The first call on a

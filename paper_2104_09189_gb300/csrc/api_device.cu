@@ -447,6 +447,7 @@ FastArgs make_fast_args(const sl_mesh *m, const FastProb *fp, const void *vin, v
     // walk itself
     a.jump = m->opt_strategy == 0 && m->opt_walk_cap == 0 ? (const int4 *)m->d.jump : nullptr;
     a.t0_init = m->d.t0_init;
+    a.initial = m->t0_initial;
     a.wq = (int4 *)m->d.wq;
     if (m->precision == SL_FP64) a.wt = (float4 *)m->d.wt;
     else a.wt2 = (float *)m->d.wt;
@@ -501,6 +502,7 @@ static void fill_fast_one(const sl_mesh *m, int32_t p, const ProbStep &q, FastPr
     double c[6] = {0, 0, 0, 0, 0, 0};
     switch (q.kind) {
     case SL_FIELD_AFFINE:
+        f.dc = make_float2((float)(q.dt * q.p[3] * q.dt), (float)(q.dt * q.p[7] * q.dt));
         c[0] = q.dt * (q.p[0] + q.p[3] * q.t);
         c[1] = q.dt * q.p[1];
         c[2] = q.dt * q.p[2];
@@ -513,15 +515,19 @@ static void fill_fast_one(const sl_mesh *m, int32_t p, const ProbStep &q, FastPr
         c[1] = q.p[1];
         c[2] = q.p[2];
         break;
-    case SL_FIELD_SWIRL: c[0] = q.dt * q.c[0]; break;
+    case SL_FIELD_SWIRL:
+        c[0] = q.dt * q.c[0];
+        f.dc.x = (float)(c[0] - q.dt * std::cos(pi * (q.t - q.dt) / q.p[0]));
+        break;
     case SL_FIELD_PAPER:
-        c[0] = q.dt * std::cos(q.p[1] * q.t);
-        c[1] = q.dt * std::sin(q.p[1] * q.t);
+    case SL_FIELD_FOURIER8: {
+        const double w = q.kind == SL_FIELD_PAPER ? q.p[1] : 2.0 * pi;
+        c[0] = q.dt * std::cos(w * q.t);
+        c[1] = q.dt * std::sin(w * q.t);
+        f.dc = make_float2((float)(c[0] - q.dt * std::cos(w * (q.t - q.dt))),
+                           (float)(c[1] - q.dt * std::sin(w * (q.t - q.dt))));
         break;
-    case SL_FIELD_FOURIER8:
-        c[0] = q.dt * std::cos(2.0 * pi * q.t);
-        c[1] = q.dt * std::sin(2.0 * pi * q.t);
-        break;
+    }
     default: break;
     }
     pack_fast_constants(q.kind, c, f);
@@ -879,6 +885,7 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
             for (int32_t k = 0; k < n_steps; ++k) {
                 FastArgs args = make_fast_args(m, (const FastProb *)((char *)m->d.fprobs + fper * k), a, b, nullptr,
                                                fh.data() + (size_t)k * m->n_problems);
+                args.initial = first_initial && k == 0;
                 args.io = (in && k == 0 ? kIoIn : 0) | (out && k == n_steps - 1 ? kIoOut : 0);
                 sl_status st = all_steady ? launch_steady(m, args, config_of(k), k, q)
                                           : launch_fast(m, args, false, config_of(k), k == 0 && first_initial, q,
@@ -899,6 +906,7 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
             if (fast) {
                 FastArgs args = make_fast_args(m, (const FastProb *)((char *)m->d.fprobs + fper * k), a, b, nullptr,
                                                fh.data() + (size_t)k * m->n_problems);
+                args.initial = first_initial && k == 0;
                 st = all_steady ? launch_steady(m, args, config_of(k), k, q)
                                 : launch_fast(m, args, false, config_of(k), k == 0 && first_initial, q, &split_seq,
                                               k > 0);

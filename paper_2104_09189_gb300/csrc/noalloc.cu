@@ -10,7 +10,7 @@
 //
 // The step reads the caller's doubles and writes doubles itself, so it needs
 // no value scratch, and a single problem's constants are kernel parameters.
-// Only a batch's constants have a home here: kNoAllocMaxProblems records (16
+// Only a batch's constants have a home here: kNoAllocMaxProblems records (18
 // KiB) in a static device array, held by every GPU that loads this library
 // until the process exits, written from the parameters of a small kernel.
 // Calls with several problems share it, so such calls that overlap on the GPU

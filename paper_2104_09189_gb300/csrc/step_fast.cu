@@ -182,7 +182,7 @@ void launch_from_df(const float2 *src, double *dst, int64_t n, cudaStream_t s)
 }
 
 namespace {
-constexpr int kConstChunk = 63;     // 4 KiB of parameters
+constexpr int kConstChunk = 56;     // 4 KiB of parameters
 struct ConstChunk {
     FastProb *dst;
     int32_t count;

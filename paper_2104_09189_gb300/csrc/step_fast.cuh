@@ -29,6 +29,8 @@ struct FastProb {
     int32_t jump_g;     // cells per side of the problem's jump table
     int32_t jump_off;   // its first cell in FastArgs::jump
     float2 c[6];        // (hi, lo)
+    float2 dc;          // how far a foot moves from one step to this one (foot_moves): table fields the
+                        // change of c0 and c1, AFFINE the change of c0 and c3 (both within 2^-20)
 };
 
 constexpr int32_t kFastCentreGrid = 1;
@@ -75,6 +77,7 @@ struct FastArgs {
     const FastProb *probs;
     FastProb prob0;               // single: a copy of probs[0] (kernel parameter space)
     int32_t single;               // one problem, prob0 valid
+    int32_t initial;              // T^0 holds the initial triangles: a foot is its displacement away
     const int64_t *node_off;
     const int2 *chunk_prob;       // more than one problem: per 128 nodes, the first and last node's
                                   // problem (chunk_problem); else NULL
@@ -137,6 +140,18 @@ constexpr float kJumpFar = 3.0f;
 __device__ __forceinline__ bool jump_far(float dx, float dy, const FastProb &P)
 {
     return (fabsf(dx) + fabsf(dy)) * (float)P.jump_g > kJumpFar;
+}
+// The same before anything of T^0 is read, by the distance (L1) the foot has
+// moved since the step before: T^0 is the triangle of the foot it moved from.
+// Nothing of T^0 is then read, a round trip and 16 bytes per node less.  With
+// 0.5, 1 and 2 cells (a cell of the table is two of the mesh wide): FP32 swirl
+// on 4.2 M nodes 2.42, 2.44 and 2.49 ms per 20 steps (2.83 without), 2.8 M nodes
+// in a batch 3.77, 3.80 and 3.86 ms per 50 (3.97), 1.05 M node swirl 0.945,
+// 0.945 and 0.962 ms (1.01); feet that stay, the same within 1 %.
+constexpr float kJumpMoves = 0.5f;
+__device__ __forceinline__ bool jump_moves(float moved, const FastProb &P)
+{
+    return moved * (float)P.jump_g > kJumpMoves;
 }
 __device__ __forceinline__ int4 jump_start(const FastArgs &a, const FastProb &P, float x, float y)
 {
@@ -202,7 +217,7 @@ void launch_gather_probe(const float4 *xyq, const int4 *t0v, const float2 *vin, 
                          cudaStream_t s);
 
 // n per-problem constants (host) to dst (device) in the parameters of a small
-// kernel, 63 per launch: dst is written in stream order and src is not read
+// kernel, 56 per launch: dst is written in stream order and src is not read
 // after the call
 void launch_put_constants(const FastProb *src, int32_t n, FastProb *dst, cudaStream_t s);
 

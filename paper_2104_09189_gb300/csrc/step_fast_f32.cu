@@ -33,9 +33,13 @@ namespace sl {
 //   FOURIER8
 // with c_k = fl32 of the per-step constants and g = fl32 of the double node
 // tables.
+// kMoved: *moved = how far (L1, about) the foot is from where T^0 was found
+// (FastProb::dc, FastArgs::initial).
+template <bool kMoved = false>
 __device__ __forceinline__ void foot_f32(const FastProb &P, const FastArgs &a, int64_t i, float x, float y, float &X,
-                                         float &Y)
+                                         float &Y, float *moved = nullptr)
 {
+    if (kMoved) *moved = 0.0f;
     const float c0 = P.c[0].x, c1 = P.c[1].x, c2 = P.c[2].x;
     switch (P.kind) {
     case SL_FIELD_AFFINE: {
@@ -44,6 +48,7 @@ __device__ __forceinline__ void foot_f32(const FastProb &P, const FastArgs &a, i
         const float fy = __fadd_rn(__fadd_rn(c3, __fmul_rn(c4, x)), __fmul_rn(c5, y));
         X = __fsub_rn(x, fx);
         Y = __fsub_rn(y, fy);
+        if (kMoved) *moved = fabsf(P.dc.x) + fabsf(P.dc.y);
         break;
     }
     case SL_FIELD_ROTATION:
@@ -54,6 +59,7 @@ __device__ __forceinline__ void foot_f32(const FastProb &P, const FastArgs &a, i
         const float2 g = a.g1f[i];
         X = __fsub_rn(x, __fmul_rn(c0, g.x));
         Y = __fsub_rn(y, __fmul_rn(c0, g.y));
+        if (kMoved) *moved = fabsf(P.dc.x) * (fabsf(g.x) + fabsf(g.y));
         break;
     }
     case SL_FIELD_PAPER:
@@ -61,6 +67,7 @@ __device__ __forceinline__ void foot_f32(const FastProb &P, const FastArgs &a, i
         const float2 g = a.g1f[i], q = a.g2f[i];
         X = __fsub_rn(x, __fadd_rn(__fmul_rn(c0, g.x), __fmul_rn(c1, q.x)));
         Y = __fsub_rn(y, __fadd_rn(__fmul_rn(c0, g.y), __fmul_rn(c1, q.y)));
+        if (kMoved) *moved = fabsf(P.dc.x * g.x + P.dc.y * q.x) + fabsf(P.dc.x * g.y + P.dc.y * q.y);
         break;
     }
     default:
@@ -472,7 +479,9 @@ __device__ __forceinline__ bool lean_node_f32(const FastArgs &a, int64_t i, int 
     const float *vin = (const float *)a.vin;
     const float2 xf = a.xyf[i];
     float X, Y;
-    foot_f32(P, a, i, xf.x, xf.y, X, Y);
+    float moves;
+    foot_f32<true>(P, a, i, xf.x, xf.y, X, Y, &moves);
+    if (a.initial) moves = fabsf(X - xf.x) + fabsf(Y - xf.y);
     if (!(X >= 0.0f && X <= 1.0f && Y >= 0.0f && Y <= 1.0f)) {
         if (kExt && a.exclude) {
             ((float *)a.vout)[i] = vin[i];
@@ -483,10 +492,16 @@ __device__ __forceinline__ bool lean_node_f32(const FastArgs &a, int64_t i, int 
         X = __double2float_rn(cx);
         Y = __double2float_rn(cy);
     }
-    int4 tq = kExt && a.grid_M > 0 ? __ldg(&a.grid_t0v[grid_slot(X, Y, a.grid_M)]) : a.t0v[i];
     // (a foot that is its node lies in all the node's triangles: walked from T^0)
     const bool jump_ok = a.jump && !(X == xf.x && Y == xf.y);
     bool moved = false, jumped = false;
+    int4 tq;
+    if (jump_ok && jump_moves(moves, P)) {
+        tq = jump_start(a, P, X, Y);
+        moved = jumped = true;
+    } else {
+        tq = kExt && a.grid_M > 0 ? __ldg(&a.grid_t0v[grid_slot(X, Y, a.grid_M)]) : a.t0v[i];
+    }
     float a0x, a0y, a1x, a1y, a2x, a2y, o1, o2, o3;
     for (;;) {
         // the triangle's vertices in slot order relative to the foot, and the

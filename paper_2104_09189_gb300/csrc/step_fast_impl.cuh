@@ -101,14 +101,16 @@ __device__ __forceinline__ bool clip_df(df x, df y, df &X, df &Y)
 // Displacement d = -dt f(x, t_{n+1}) of the Euler foot X = x + d (Eq. 4) in
 // double-float, with the field's time factors folded into the per-step
 // constants.
-template <int kKind>
+// kMoved: *moved = the change of the displacement since the step before (L1).
+template <int kKind, bool kMoved = false>
 __device__ __forceinline__ void disp_df_k(const FastProb &P, const FastArgs &a, int64_t i, df x, df y, df &DX,
-                                          df &DY)
+                                          df &DY, float *moved = nullptr)
 {
     switch (kKind) {
     case SL_FIELD_AFFINE: {
         DX = df_neg(df_add(df_add(dfp(P.c[0]), df_mul(dfp(P.c[1]), x)), df_mul(dfp(P.c[2]), y)));
         DY = df_neg(df_add(df_add(dfp(P.c[3]), df_mul(dfp(P.c[4]), x)), df_mul(dfp(P.c[5]), y)));
+        if (kMoved) *moved = fabsf(P.dc.x) + fabsf(P.dc.y);
         break;
     }
     case SL_FIELD_ROTATION:
@@ -129,6 +131,7 @@ __device__ __forceinline__ void disp_df_k(const FastProb &P, const FastArgs &a, 
         const df k = dfp(P.c[0]);
         DX = df_neg(df_mul(k, df_make(g.x, g.z)));
         DY = df_neg(df_mul(k, df_make(g.y, g.w)));
+        if (kMoved) *moved = fabsf(P.dc.x) * (fabsf(g.x) + fabsf(g.y));
         break;
     }
     case SL_FIELD_PAPER:
@@ -137,6 +140,7 @@ __device__ __forceinline__ void disp_df_k(const FastProb &P, const FastArgs &a, 
         const df k0 = dfp(P.c[0]), k1 = dfp(P.c[1]);
         DX = df_neg(df_add(df_mul(k0, df_make(g.x, g.z)), df_mul(k1, df_make(q.x, q.z))));
         DY = df_neg(df_add(df_mul(k0, df_make(g.y, g.w)), df_mul(k1, df_make(q.y, q.w))));
+        if (kMoved) *moved = fabsf(P.dc.x * g.x + P.dc.y * q.x) + fabsf(P.dc.x * g.y + P.dc.y * q.y);
         break;
     }
     default:
@@ -147,15 +151,17 @@ __device__ __forceinline__ void disp_df_k(const FastProb &P, const FastArgs &a, 
 }
 
 // The same for a kind known only at run time.
-__device__ __forceinline__ void disp_df(const FastProb &P, const FastArgs &a, int64_t i, df x, df y, df &DX, df &DY)
+template <bool kMoved = false>
+__device__ __forceinline__ void disp_df(const FastProb &P, const FastArgs &a, int64_t i, df x, df y, df &DX, df &DY,
+                                        float *moved = nullptr)
 {
     switch (P.kind) {
-    case SL_FIELD_AFFINE: disp_df_k<SL_FIELD_AFFINE>(P, a, i, x, y, DX, DY); break;
-    case SL_FIELD_ROTATION: disp_df_k<SL_FIELD_ROTATION>(P, a, i, x, y, DX, DY); break;
-    case SL_FIELD_SWIRL: disp_df_k<SL_FIELD_SWIRL>(P, a, i, x, y, DX, DY); break;
-    case SL_FIELD_PAPER: disp_df_k<SL_FIELD_PAPER>(P, a, i, x, y, DX, DY); break;
-    case SL_FIELD_FOURIER8: disp_df_k<SL_FIELD_FOURIER8>(P, a, i, x, y, DX, DY); break;
-    default: disp_df_k<SL_FIELD_ZERO>(P, a, i, x, y, DX, DY); break;
+    case SL_FIELD_AFFINE: disp_df_k<SL_FIELD_AFFINE, kMoved>(P, a, i, x, y, DX, DY, moved); break;
+    case SL_FIELD_ROTATION: disp_df_k<SL_FIELD_ROTATION, kMoved>(P, a, i, x, y, DX, DY, moved); break;
+    case SL_FIELD_SWIRL: disp_df_k<SL_FIELD_SWIRL, kMoved>(P, a, i, x, y, DX, DY, moved); break;
+    case SL_FIELD_PAPER: disp_df_k<SL_FIELD_PAPER, kMoved>(P, a, i, x, y, DX, DY, moved); break;
+    case SL_FIELD_FOURIER8: disp_df_k<SL_FIELD_FOURIER8, kMoved>(P, a, i, x, y, DX, DY, moved); break;
+    default: disp_df_k<SL_FIELD_ZERO, kMoved>(P, a, i, x, y, DX, DY, moved); break;
     }
 }
 
@@ -641,16 +647,20 @@ __device__ __forceinline__ void foot_to_grid(df &X, df &Y)
 // that is the node itself (an outward boundary node); a foot inside the
 // square is not reported here.  gone (kExt, with a.exclude): the foot leaves
 // the square and the node is excluded (X, Y are then not set).
-// kInside: a foot inside the square that is its node's pair is reported too.
+// kInside: a foot inside the square that is its node's pair is reported too,
+// and moved is the distance (L1, about) of the unclipped foot from where T^0 was
+// found (FastProb::dc, FastArgs::initial).
 template <int kKind, bool kExt = false, bool kInside = false>
 __device__ __forceinline__ bool foot_pair(const FastArgs &a, int64_t i, const FastProb &P, df &X, df &Y,
-                                          bool &at_node, bool &gone)
+                                          bool &at_node, bool &gone, float *moved = nullptr)
 {
     const float4 xq = a.xyq[i];
     const df x = df_make(xq.x, xq.z), y = df_make(xq.y, xq.w);
     df DX, DY;
-    if (kKind < 0) disp_df(P, a, i, x, y, DX, DY);
+    if (kInside) *moved = 0.0f;
+    if (kKind < 0) disp_df<kInside>(P, a, i, x, y, DX, DY, moved);
     else disp_df_k<kKind < 0 ? 0 : kKind>(P, a, i, x, y, DX, DY);
+    if (kInside && a.initial) *moved = fabsf(DX.h) + fabsf(DY.h);
     at_node = false;
     gone = false;
     if (foot_grid(x, DX, X) & foot_grid(y, DY, Y)) {

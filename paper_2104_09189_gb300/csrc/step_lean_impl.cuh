@@ -117,13 +117,21 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
     }
     df X, Y;
     bool at_node, gone;
-    const bool clipped = foot_pair<-1, kExt, true>(a, i, P, X, Y, at_node, gone);
+    float moves;
+    const bool clipped = foot_pair<-1, kExt, true>(a, i, P, X, Y, at_node, gone, &moves);
     const float2 *vin = (const float2 *)a.vin;
     if (kExt && gone) {
         keep_value(a, i);
         return true;
     }
-    int4 tq = kExt && a.grid_M > 0 ? __ldg(&a.grid_t0v[grid_slot(X.h, Y.h, a.grid_M)]) : a.t0v[i];
+    bool moved = false, jumped = false;
+    int4 tq;
+    if (a.jump && !at_node && jump_moves(moves, P)) {
+        tq = jump_start(a, P, X.h, Y.h);
+        moved = jumped = true;
+    } else {
+        tq = kExt && a.grid_M > 0 ? __ldg(&a.grid_t0v[grid_slot(X.h, Y.h, a.grid_M)]) : a.t0v[i];
+    }
     if (at_node) {
         // the foot is its own node: see step_node
         if (tq.y != (int32_t)i && tq.z != (int32_t)i && tq.w != (int32_t)i) return false;
@@ -132,7 +140,6 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
         return true;
     }
     float4 A = a.xyq[tq.y], B = a.xyq[tq.z], C = a.xyq[tq.w];
-    bool moved = false, jumped = false;
     for (;;) {
         const int k = outside_edge(A, B, C, X.h, Y.h);
         if (k < 0) break;
