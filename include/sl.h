@@ -139,7 +139,9 @@ typedef enum {
                                 128x9, 256x5, 128x12 (default 5) */
     SL_OPT_CONFIG_FIRST = 7, /* launch configuration for a step whose walks start at the initial
                                 incident triangles (the first step after sl_mesh_create or
-                                sl_mesh_reset_t0): long walks favour fewer resident warps (default 0) */
+                                sl_mesh_reset_t0): long walks favour fewer resident warps (default 0;
+                                until it is set, a first step that may start at the table of start
+                                triangles, see SL_OPT_WALK_CAP, takes SL_OPT_CONFIG's) */
     SL_OPT_STRATEGY = 8,     /* start triangle of the walks (Sec. 3): 0 = strategy (b), the triangle
                                 found at the previous step (default); 1 = strategy (a), the node's own
                                 incident triangle at every step (T^0 is never overwritten); 2 = the

@@ -842,7 +842,7 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
         g.t0_initial = first_initial;
         g.split = m->opt_split;
     };
-    auto config_of = [&](int32_t k) { return (k == 0 && first_initial) ? m->opt_config_first : m->opt_config; };
+    auto config_of = [&](int32_t k) { return (k == 0 && first_initial) ? first_config(m) : m->opt_config; };
     std::vector<FastProb> fh;   // the fast kernels' constants, host copy (filled when recording)
     bool all_steady = false;
     if (!reuse) {
@@ -1021,7 +1021,7 @@ extern "C" sl_status sl_step(sl_mesh *m, const sl_problem *probs, int64_t n, con
     } else {
         FastArgs a = make_fast_args(m, (const FastProb *)m->d.fprobs, v_in, v_out, dbg, fh.data());
         if (m->precision == SL_FP64) a.io = kIoIn | kIoOut;
-        st = launch_fast(m, a, debug, m->t0_initial ? m->opt_config_first : m->opt_config, m->t0_initial, s);
+        st = launch_fast(m, a, debug, m->t0_initial ? first_config(m) : m->opt_config, m->t0_initial, s);
         if (st != SL_OK) return st;
     }
     m->stepped = true;
