@@ -116,17 +116,44 @@ SL_HD OrientResult orient(double ax, double ay, double bx, double by, double cx,
 // Exact orientation on the device in integers.  A coordinate in [-1, 1] that
 // is a multiple of 2^-62 (every double of at least 2^-9 is one, and every
 // float of at least 2^-38) is an int64 in those units; differences of two
-// in [0, 1] stay below 2^62 and the two products of an orientation below
-// 2^124, so the sign is that of a difference of two 128-bit products.  This
-// takes about a hundred cycles where the floating-point expansions above
-// run a chain of dependent FP64 operations for 25 us, which a whole step waits
-// for: on a Courant grid of 1 M nodes with 78 feet on grid lines per step, a
-// step of 57 us became one of 40 us (20 of them 1.14 -> 0.81 ms).
+// in [0, 1] stay within 2^62 and the two products of an orientation within
+// 2^124, so the sign is that of a difference of two 128-bit products.
+// What this saves is latency, which a whole step waits for when a few feet lie
+// on grid lines: the expansion above takes 13 000 cycles per edge (one FP64
+// operation about 180), three edges in integers 1 800, or 3 500 when the
+// coordinates are converted on the FP64 pipe instead of by shifts.  20 steps
+// with 78 such feet each on 1 M nodes 1.14 -> 0.74 ms (0.81 with FP64
+// conversions), a batch of 64 meshes 3.77 -> 3.68 ms per 50 steps by the shifts.
 __device__ __forceinline__ bool fixed62(double v, long long &n)
 {
-    const double s = v * 0x1p62;
-    n = __double2ll_rn(s);
-    return fabs(v) <= 1.0 && (double)n == s;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7FFu);
+    const long long m = (long long)(b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ll;     // v = m 2^(e - 1075)
+    const int s = e - (1075 - 62);                                                   // n = m 2^s
+    if ((b << 1) == 0) {
+        n = 0;
+        return true;
+    }
+    n = s >= 0 ? m << (s & 63) : m >> ((-s) & 63);
+    const bool ok = s <= 10 && s > -53 && (s >= 0 || n << ((-s) & 63) == m);             // |v| < 2, no bit lost
+    if (b >> 63) n = -n;
+    return ok;
+}
+
+__device__ __forceinline__ bool fixed62(float v, long long &n)
+{
+    const unsigned int b = __float_as_uint(v);
+    const int e = (int)((b >> 23) & 0xFFu);
+    const long long m = (long long)(b & 0x7FFFFFu) | 0x800000ll;                        // v = m 2^(e - 150)
+    const int s = e - (150 - 62);
+    if ((b << 1) == 0) {
+        n = 0;
+        return true;
+    }
+    n = s >= 0 ? m << (s & 63) : m >> ((-s) & 63);
+    const bool ok = s <= 39 && s > -24 && (s >= 0 || n << ((-s) & 63) == m);
+    if (b >> 31) n = -n;
+    return ok;
 }
 
 // Sign of (q - p) x (x - p) for points in [0, 1]^2 in units of 2^-62.

@@ -264,21 +264,21 @@ __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int 
                 // conversions of the loop-invariant foot inside it
                 const int32_t jj = tri_of_f32(e0), sa = e0 - 3 * jj, sb = e1 - 3 * jj, sc = 3 - sa - sb;
                 const float2 A = a.xyf[a.tv[sa][jj]], B = a.xyf[a.tv[sb][jj]], C = a.xyf[a.tv[sc][jj]];
-                float xb = X, yb = Y;
-                asm volatile("" : "+f"(xb), "+f"(yb));
-                const double Xd = xb, Yd = yb;
                 if (!kCount) {
                     // integers where the coordinates allow (the counting variants
                     // take the stages below, which give the same signs)
                     long long ax, ay, bx, by, cx, cy, x, y;
                     if (slp::fixed62(A.x, ax) & slp::fixed62(A.y, ay) & slp::fixed62(B.x, bx) &
-                        slp::fixed62(B.y, by) & slp::fixed62(C.x, cx) & slp::fixed62(C.y, cy) & slp::fixed62(Xd, x) &
-                        slp::fixed62(Yd, y)) {
+                        slp::fixed62(B.y, by) & slp::fixed62(C.x, cx) & slp::fixed62(C.y, cy) & slp::fixed62(X, x) &
+                        slp::fixed62(Y, y)) {
                         if (s1 == 2) s1 = slp::orient_fixed62(bx, by, cx, cy, x, y);
                         if (s2 == 2) s2 = slp::orient_fixed62(cx, cy, ax, ay, x, y);
                         if (s3 == 2) s3 = slp::orient_fixed62(ax, ay, bx, by, x, y);
                     }
                 }
+                float xb = X, yb = Y;
+                asm volatile("" : "+f"(xb), "+f"(yb));
+                const double Xd = xb, Yd = yb;
                 if (s1 == 2) {
                     slp::OrientResult r = slp::orient(B.x, B.y, C.x, C.y, Xd, Yd);
                     s1 = r.sign;
