@@ -83,6 +83,7 @@ struct FastArgs {
                                   // problem (chunk_problem); else NULL
     int32_t nprob;
     int32_t walk_cap;
+    int32_t capped;               // host side: walk_cap is the caller's (the full node step keeps to it)
     int64_t N;
     uint32_t *status;
     unsigned long long *stats;
@@ -159,15 +160,6 @@ __device__ __forceinline__ int4 jump_start(const FastArgs &a, const FastProb &P,
     return __ldg(&a.jump[P.jump_off + jump_cell(y, g) * g + jump_cell(x, g)]);
 }
 
-// A foot found in triangle j with these signs (none negative, at least one
-// zero) lies on a vertex or on an edge between two triangles; a zero on one
-// edge of the boundary alone leaves j the only triangle.
-__device__ __forceinline__ bool shared_zero(const FastArgs &a, int32_t j, int s1, int s2, int s3)
-{
-    if ((s1 == 0) + (s2 == 0) + (s3 == 0) > 1) return true;
-    return a.tn[s1 == 0 ? 0 : (s2 == 0 ? 1 : 2)][j] >= 0;
-}
-
 template <typename Kernel>
 inline void launch_step_kernel(Kernel k, unsigned grid, unsigned block, cudaStream_t s, const FastArgs &a)
 {
@@ -199,7 +191,7 @@ void launch_lean_df_c3(const FastArgs &a, cudaStream_t s);
 void launch_lean_df_c4(const FastArgs &a, cudaStream_t s);
 void launch_lean_df_c5(const FastArgs &a, cudaStream_t s);
 void launch_lean_df_ext(const FastArgs &a, cudaStream_t s);
-// the full node step alone: statistics, debug outputs, strategy (c)
+// the full node step alone: statistics, debug outputs, strategy (c), a hop cap
 void launch_full_df(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
 // the two passes of a split step: lean settle pass, then the finish pass over
 // its queue (reset: zero the queue counter first)

@@ -152,6 +152,10 @@ template <bool kDebug, bool kCount, bool kExt>
 __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int pi, CountersF32 &c)
 {
     const FastProb &P = a.single ? a.prob0 : a.probs[pi];
+    if (!kCount && (P.flags & kFastUse)) {
+        apply_weights_f32(a, i);
+        return;
+    }
     const float2 xf = a.xyf[i];
     float X, Y;
     foot_f32(P, a, i, xf.x, xf.y, X, Y);
@@ -645,18 +649,18 @@ static void launch_f32_cfg(const FastArgs &a, bool stats, bool debug, cudaStream
         else launch_step_kernel(k_step_fast_f32<true, false, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
     } else {
         if (debug) launch_step_kernel(k_step_fast_f32<false, true, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
-        else if constexpr (kExt)    // strategy (c); the lean kernel takes the others
+        else if constexpr (kExt)    // strategy (c), a hop cap; the lean kernel takes the others
             launch_step_kernel(k_step_fast_f32<false, false, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
     }
 }
 
 void launch_fast_f32(const FastArgs &a, bool stats, bool debug, int config, cudaStream_t s)
 {
-    // statistics, debug outputs and strategy (c): the full node step, one
-    // configuration (128 x 8)
+    // statistics, debug outputs, a hop cap of the caller's and strategy (c): the
+    // full node step, one configuration (128 x 8)
     const bool ext = a.exclude || a.order || a.grid_M > 0 || a.keep_t0;
-    if (stats || debug || a.order) {
-        if (ext) launch_f32_cfg<128, 8, true>(a, stats, debug, s);
+    if (stats || debug || a.order || a.capped) {
+        if (ext || !(stats || debug)) launch_f32_cfg<128, 8, true>(a, stats, debug, s);
         else launch_f32_cfg<128, 8>(a, stats, debug, s);
         return;
     }

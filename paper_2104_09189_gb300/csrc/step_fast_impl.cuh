@@ -909,6 +909,10 @@ template <bool kDebug, bool kCount, bool kExt, bool kCompact>
 __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, NodeCounters &c)
 {
     const FastProb &P = a.single ? a.prob0 : a.probs[pi];
+    if (!kCount && (P.flags & kFastUse)) {
+        put_value(a, i, apply_weights(a, i));
+        return;
+    }
     const float4 xq = a.xyq[i];
     const df x = df_make(xq.x, xq.z), y = df_make(xq.y, xq.w);
     df DX, DY;
@@ -1400,7 +1404,7 @@ inline void launch_fast_df_form(const FastArgs &a, bool stats, bool debug, unsig
         else launch_step_kernel(k_step_fast_df<true, false, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
     } else {
         if (debug) launch_step_kernel(k_step_fast_df<false, true, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
-        else if constexpr (kExt)    // strategy (c); the lean kernel takes the others
+        else if constexpr (kExt)    // strategy (c), a hop cap; the lean kernel takes the others
             launch_step_kernel(k_step_fast_df<false, false, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
     }
 }

@@ -118,6 +118,26 @@ def test_exact_signs_near_a_corner(scale, precision):
         v = q
 
 
+@pytest.mark.parametrize("precision", [sl.SL_FP64, sl.SL_FP32], ids=["fp64", "fp32"])
+def test_a_hop_cap_holds_without_counting(precision):
+    """A cap of the caller's ends a walk that needs more hops (and its fallback)
+    whether or not the step counts or reports."""
+    m = si.grid_mesh(40, 0.25, 2)
+    f = si.affine_field([0.02 * 10, 0, 0, 0, 0, 0, 0, 0])      # 4 cells: 8 to 10 hops
+    for cap, ok in ((1, False), (2, False), (64, True)):
+        g = DeviceRun(m, f, 0.5, precision=precision)
+        sl.sl_mesh_set_option(g.h, sl.SL_OPT_WALK_CAP, cap)
+        v = g.to_dev(si.gaussian(m.xy))
+        w = g.torch.empty_like(v)
+        sl.sl_step(g.h, g.probs, 0, v, w)
+        if ok:
+            sl.sl_mesh_status(g.h)
+        else:
+            with pytest.raises(sl.SLError) as e:
+                sl.sl_mesh_status(g.h)
+            assert e.value.status == sl.SL_E_WALK_LIMIT
+
+
 def test_jump_table_of_uneven_batch():
     """Meshes of 9 to 10 000 nodes in one batch, each with a table of its own."""
     import torch
