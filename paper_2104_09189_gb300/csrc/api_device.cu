@@ -113,7 +113,7 @@ void free_device(sl_mesh *m)
 {
     release_l2_window(m);
     DeviceMesh &d = m->d;
-    void *ptrs[] = {d.xy, d.tv[0], d.tv[1], d.tv[2], d.tn[0], d.tn[1], d.tn[2], d.t0, d.t0_init, d.t0v, d.node_off, d.chunk_prob,
+    void *ptrs[] = {d.xy, d.tv[0], d.tv[1], d.tv[2], d.tn[0], d.tn[1], d.tn[2], d.t0, d.t0_init, d.pair_tri, d.t0v, d.node_off, d.chunk_prob,
                     d.status, d.probs, d.fprobs, d.xyq, d.xyh, d.g1, d.g2, d.tparams, d.dfa, d.dfb, d.he, d.he8, d.wq, d.wt, d.tri, d.jump, d.grid_t0v, d.tree_order, d.tree_parent, d.queue, d.queue_count,
                     m->host_v, m->host_v2};
     for (void *p : ptrs)
@@ -228,6 +228,11 @@ static sl_status upload_arrays(sl_mesh *m)
     }
     st = build_jump_table(m);
     if (st != SL_OK) return st;
+    if (m->precision == SL_FP64) {
+        if (!d.pair_tri) SL_CUDA(cudaMalloc(&d.pair_tri, sizeof(int32_t) * N));
+        launch_pair_tri(make_fast_args(m, nullptr, nullptr, nullptr, nullptr), d.pair_tri, 0);
+        SL_CUDA(cudaGetLastError());
+    }
     launch_fill_t0v(d.t0, d.tv[0], d.tv[1], d.tv[2], (int4 *)d.t0v, N, 0);
     SL_CUDA(cudaGetLastError());
     SL_CUDA(cudaDeviceSynchronize());
@@ -447,6 +452,7 @@ FastArgs make_fast_args(const sl_mesh *m, const FastProb *fp, const void *vin, v
     // walk itself
     a.jump = m->opt_strategy == 0 && m->opt_walk_cap == 0 ? (const int4 *)m->d.jump : nullptr;
     a.t0_init = m->d.t0_init;
+    a.pair_tri = m->d.pair_tri;
     a.initial = m->t0_initial;
     a.wq = (int4 *)m->d.wq;
     if (m->precision == SL_FP64) a.wt = (float4 *)m->d.wt;

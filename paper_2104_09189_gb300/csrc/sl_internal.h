@@ -33,6 +33,7 @@ struct DeviceMesh {
                                                     // boundary: -1 - side (0: x=0, 1: x=1, 2: y=0, 3: y=1)
     int32_t *t0 = nullptr;            // start / last foot triangle of node i (global)
     int32_t *t0_init = nullptr;       // the initial start triangles (global)
+    int32_t *pair_tri = nullptr;      // FP64: the triangle of each node's coordinate pair, or -1
     void *t0v = nullptr;              // int4 (T^0, its vertex ids) per node
     void *grid_t0v = nullptr;         // int4 start state per structured-grid triangle (strategy 2)
     int32_t *queue = nullptr;         // split steps: nodes left to the finish pass (N)

@@ -123,6 +123,44 @@ void launch_apply_df(const FastArgs &a, cudaStream_t s)
     if (grid) launch_step_kernel(k_apply_df, grid, 256, s, a);
 }
 
+// The triangle that holds node i's coordinate pair, the point a foot of no
+// displacement (or one below the pair's rounding) is: within 2^-49 of the node,
+// so among the node's triangles, found from the initial one over negative
+// exact signs.  -1: the pair is on a vertex or between two triangles, where the
+// step's own path decides.  Once per mesh and numbering, for the full step's
+// foot_on_pair: with exact signs for every node of a step at which the field
+// vanishes, and for a third of a swirl's boundary nodes at every step, 20 steps
+// on 1.05 M nodes took 1.005 ms, 0.910 without; 1.18 M node-steps in two calls
+// 70 -> 66 us.  (Asked in the lean pass instead it cost that pass 2 to 8 %.)
+__global__ void k_pair_tri(const __grid_constant__ FastArgs a, int32_t *__restrict__ pair_tri)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= a.N) return;
+    const float4 xq = a.xyq[i];
+    const df X = df_make(xq.x, xq.z), Y = df_make(xq.y, xq.w);
+    int32_t j = a.t0_init[i], found = -1;
+    for (int hop = 0; hop < 64; ++hop) {
+        const uint32_t r = exact_signs<false>(a.xyd, a.tv[0][j], a.tv[1][j], a.tv[2][j], X, Y, 7u);
+        if (r & (1u << 12)) break;                       // a coordinate outside the exact range
+        if (r & 0x2au) {
+            const int32_t u = a.tn[r & 2u ? 0 : (r & 8u ? 1 : 2)][j];
+            if (u < 0) break;
+            j = u;
+            continue;
+        }
+        const uint32_t pos = r & 0x15u;
+        const int zeros = 3 - __popc(pos), k = !(pos & 1u) ? 0 : (!(pos & 4u) ? 1 : 2);
+        if (zeros == 0 || (zeros == 1 && a.tn[k][j] < 0)) found = j;
+        break;
+    }
+    pair_tri[i] = found;
+}
+
+void launch_pair_tri(const FastArgs &a, int32_t *pair_tri, cudaStream_t s)
+{
+    if (a.N > 0) k_pair_tri<<<(unsigned)((a.N + 127) / 128), 128, 0, s>>>(a, pair_tri);
+}
+
 // ---------------------------------------------------------------------------
 // Gather probe: the memory accesses of a step whose feet stay in their start
 // triangles, with only a sum as arithmetic (sl_probe_gather).

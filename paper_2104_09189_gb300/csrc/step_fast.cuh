@@ -61,6 +61,8 @@ struct FastArgs {
     // start at T^0 only
     const int4 *jump;
     const int32_t *t0_init;       // the node's initial incident triangle
+    const int32_t *pair_tri;      // FP64 meshes: the triangle that holds the node's coordinate pair (not its
+                                  // double coordinates), or -1 when there are several
     int32_t *t0;
     int4 *t0v;                    // per node: (3 T^0, T[0][T^0], T[1][T^0], T[2][T^0]), kept in
                                   // step with t0
@@ -281,6 +283,9 @@ void launch_build_jump(const JumpBuildArgs &a, cudaStream_t s);
 
 // tri[t] = (3 t, its three vertex ids in slot order)
 void launch_build_tri(const int32_t *const tv[3], int64_t nt, int4 *tri, cudaStream_t s);
+
+// pair_tri (FastArgs) from the mesh arrays of a: xyq, xyd, tv, tn, t0_init, N
+void launch_pair_tri(const FastArgs &a, int32_t *pair_tri, cudaStream_t s);
 
 // t0v[i] = (3 t0[i], its three vertex ids in slot order)
 void launch_fill_t0v(const int32_t *t0, const int32_t *tv0, const int32_t *tv1, const int32_t *tv2, int4 *t0v,

@@ -300,51 +300,6 @@ __device__ __forceinline__ int unpack_sign(uint32_t r, int k)
     return v == 1u ? 1 : (v == 2u ? -1 : 0);
 }
 
-// Signs of the edges selected by `need` (as exact_signs) for a foot that came
-// out of the foot arithmetic as node i's own pair, in a triangle with node i
-// as a vertex.  The foot is then node i + d exactly, d = pair - double
-// coordinate (|d| <= 2^-49, exact in float for all but tiny coordinates), and
-// an edge P -> Q through node i has orient(P, Q, foot) = (Q - P) x d exactly:
-// no cancellation is left and float decides it.  With Q - P rounded from the
-// pair form (within 2^-24 relative and 2^-47 absolute of the exact
-// difference) the float cross product is within 2^-21 of the |.|-sum of its
-// products plus 2^-46 |d|_1; a sign inside that bound, or an edge not through
-// node i, stays undecided.  Returns the packed signs and, in bits 8..10, the
-// edges still undecided.  Where a field vanishes at a whole time level every
-// node comes here (the swirl's pause): with the FP64 stages of exact_signs that
-// step took 1.53 ms on 1.05 M nodes, the steps around it 0.05 ms, and a run
-// of 20 steps 2.52 ms; 1.21 ms with this.
-static __device__ __noinline__ uint32_t node_signs(const double2 *__restrict__ xyd, int i, int w0, int w1, int w2,
-                                                   float4 A, float4 B, float4 C, df X, df Y, uint32_t need)
-{
-    const double2 x = xyd[i];
-    const double ex = __dsub_rn((double)X.l, __dsub_rn(x.x, (double)X.h));    // both differences are exact
-    const double ey = __dsub_rn((double)Y.l, __dsub_rn(x.y, (double)Y.h));
-    const float dx = __double2float_rn(ex), dy = __double2float_rn(ey);
-    const float dd = fabsf(dx) + fabsf(dy);
-    // (below 2^-90 the products come near the subnormals)
-    if ((double)dx != ex || (double)dy != ey || (dd != 0.0f && dd < 0x1p-90f)) return need << 8;
-    uint32_t out = 0, left = 0;
-    for (int k = 0; k < 3; ++k) {
-        if (!(need >> k & 1u)) continue;
-        const float4 P = k == 0 ? B : (k == 1 ? C : A), Q = k == 0 ? C : (k == 1 ? A : B);
-        const int p = k == 0 ? w1 : (k == 1 ? w2 : w0), q = k == 0 ? w2 : (k == 1 ? w0 : w1);
-        if (p != i && q != i) {
-            left |= 1u << k;
-            continue;
-        }
-        const float qx = __fadd_rn(__fsub_rn(Q.x, P.x), __fsub_rn(Q.z, P.z));
-        const float qy = __fadd_rn(__fsub_rn(Q.y, P.y), __fsub_rn(Q.w, P.w));
-        const float t1 = __fmul_rn(qx, dy), t2 = __fmul_rn(qy, dx);
-        const float c = __fsub_rn(t1, t2), e = 0x1p-21f * (fabsf(t1) + fabsf(t2)) + 0x1p-46f * dd;
-        if (dd == 0.0f) continue;                    // the foot is the node: exactly 0
-        if (c > e) out |= 1u << (2 * k);
-        else if (c < -e) out |= 2u << (2 * k);
-        else left |= 1u << k;
-    }
-    return out | (left << 8);
-}
-
 // Randomised visibility walk step: a uniformly drawn negative edge (signs
 // s1..s3 of the edges opposite W0..W2, at least one negative).
 __device__ __forceinline__ int random_negative_edge(int64_t i, uint32_t hops, int s1, int s2, int s3)
@@ -621,6 +576,16 @@ __device__ __forceinline__ float2 apply_weights(const FastArgs &a, int64_t i)
 __device__ __forceinline__ bool foot_is_node(df x, df y, df X, df Y)
 {
     return X.h == x.h && X.l == x.l && Y.h == y.h && Y.l == y.l;
+}
+
+// X, Y, in (grid, remainder) form, is the pair x of a node (gx, gy, rx, ry):
+// the same sums, the grid parts perhaps one step of 2^-24 apart (a sum halfway
+// between two grid values).
+__device__ __forceinline__ bool foot_on_pair(float4 x, df X, df Y)
+{
+    const float dx = __fsub_rn(X.h, x.x), dy = __fsub_rn(Y.h, x.y);
+    return __fsub_rn(x.z, dx) == X.l && __fadd_rn(X.l, dx) == x.z && __fsub_rn(x.w, dy) == Y.l &&
+           __fadd_rn(Y.l, dy) == x.w;
 }
 
 // A foot with both high parts strictly inside (0, 1) needs neither the
@@ -995,13 +960,31 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     int32_t e0 = tq.x, e1 = 0;
     int32_t j = 0;
     int w0 = tq.y, w1 = tq.z, w2 = tq.w;
+    // A foot that ends as its node's coordinate pair, within rounding of the
+    // node, is a point of the mesh alone, and its triangle is known (k_pair_tri;
+    // the counting variants walk there).
+    const int32_t known = !kCount && foot_on_pair(a.xyq[i], X, Y) ? a.pair_tri[i] : -1;
     bool ids = true;           // w0..w2 are the vertex ids of the current triangle
     const uint32_t cap = (uint32_t)a.walk_cap;
     uint32_t &hops = c.hops;
     bool found = false;
     int s1 = 0, s2 = 0, s3 = 0;
     df n1, n2, den;
-    if (cap > 0) {
+    if (known >= 0) {
+        const int4 tk = a.tri[known];
+        j = known;
+        w0 = tk.y;
+        w1 = tk.z;
+        w2 = tk.w;
+        const Numerators t = numerators(a.xyq[w0], a.xyq[w1], a.xyq[w2], Xg, Xr, Yg, Yr);
+        n1 = t.n1;
+        n2 = t.n2;
+        den = t.den;
+        found = true;
+        s1 = s2 = s3 = 1;
+        hops = known != tri_of(tq.x);     // T^0 changes
+    }
+    if (!found && cap > 0) {
         // A foot that moved is usually clear of its start triangle: test the
         // three edges of T^0 in FP32 first and, when one is certainly
         // negative, hop at once (the certified test then runs where the FP32
@@ -1052,7 +1035,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
             }
         }
     }
-    for (;;) {
+    while (!found) {
         // certified test in double-float on (W0, W1, W2) = the vertices in
         // slot order, relative to W2
         j = tri_of(e0);
@@ -1089,19 +1072,8 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
             if (s3 == 2) { const int32_t nb = a.tn[2][j]; if (nb < 0 && (fside >> (-1 - nb) & 1u)) s3 = 0; }
         }
         if (s1 == 2 || s2 == 2 || s3 == 2) {
-            uint32_t need = (s1 == 2 ? 1u : 0u) | (s2 == 2 ? 2u : 0u) | (s3 == 2 ? 4u : 0u);
-            const float4 xn = a.xyq[i];
-            if (!kCount && foot_is_node(df_make(xn.x, xn.z), df_make(xn.y, xn.w), X, Y)) {
-                // the foot is the node's own pair (the counting variants take the
-                // stages below, which give the same signs)
-                const uint32_t r = node_signs(a.xyd, (int)i, w0, w1, w2, A, B, C, X, Y, need), done = need & ~(r >> 8);
-                if (done & 1u) s1 = unpack_sign(r, 0);
-                if (done & 2u) s2 = unpack_sign(r, 1);
-                if (done & 4u) s3 = unpack_sign(r, 2);
-                need &= r >> 8;
-            }
             // exact signs on the double coordinates and the exact foot
-            const uint32_t r = need ? exact_signs<kCount>(a.xyd, w0, w1, w2, X, Y, need) : 0u;
+            const uint32_t r = exact_signs<kCount>(a.xyd, w0, w1, w2, X, Y, (s1 == 2 ? 1u : 0u) | (s2 == 2 ? 2u : 0u) | (s3 == 2 ? 4u : 0u));
             if (s1 == 2) s1 = unpack_sign(r, 0);
             if (s2 == 2) s2 = unpack_sign(r, 1);
             if (s3 == 2) s3 = unpack_sign(r, 2);
