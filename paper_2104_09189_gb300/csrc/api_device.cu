@@ -403,7 +403,6 @@ static StepArgs make_args(const sl_mesh *m, const ProbStep *probs_dev, const voi
         a.tv[k] = m->d.tv[k];
         a.tn[k] = m->d.tn[k];
     }
-    a.t0 = m->d.t0;
     a.t0v = (int4 *)m->d.t0v;
     a.vin = vin;
     a.vout = vout;
@@ -457,7 +456,6 @@ FastArgs make_fast_args(const sl_mesh *m, const FastProb *fp, const void *vin, v
     a.wq = (int4 *)m->d.wq;
     if (m->precision == SL_FP64) a.wt = (float4 *)m->d.wt;
     else a.wt2 = (float *)m->d.wt;
-    a.t0 = m->d.t0;
     a.t0v = (int4 *)m->d.t0v;
     a.vin = vin;
     a.vout = vout;
@@ -1081,7 +1079,8 @@ extern "C" sl_status sl_run_host(sl_mesh *m, const sl_problem *probs, int64_t n0
 extern "C" sl_status sl_mesh_get_t0(const sl_mesh *m, int32_t *t0_dev, void *stream)
 {
     if (!m || !t0_dev) return fail(SL_E_ARG, "sl_mesh_get_t0: NULL argument");
-    SL_CUDA(cudaMemcpyAsync(t0_dev, m->d.t0, sizeof(int32_t) * m->N, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
+    launch_export_t0((const int4 *)m->d.t0v, t0_dev, m->N, (cudaStream_t)stream);
+    SL_CUDA(cudaGetLastError());
     return SL_OK;
 }
 
@@ -1095,9 +1094,8 @@ extern "C" sl_status sl_mesh_set_t0(sl_mesh *m, const int32_t *t0_dev, void *str
         for (int64_t i = m->node_off[p]; i < m->node_off[p + 1]; ++i)
             if (h[i] < m->tri_off[p] || h[i] >= m->tri_off[p + 1])
                 return fail(SL_E_ARG, "sl_mesh_set_t0: entry " + std::to_string(i) + " is not a triangle of its problem");
-    SL_CUDA(cudaMemcpyAsync(m->d.t0, t0_dev, sizeof(int32_t) * m->N, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
     m->t0_initial = false;
-    launch_fill_t0v(m->d.t0, m->d.tv[0], m->d.tv[1], m->d.tv[2], (int4 *)m->d.t0v, m->N, (cudaStream_t)stream);
+    launch_fill_t0v(t0_dev, m->d.tv[0], m->d.tv[1], m->d.tv[2], (int4 *)m->d.t0v, m->N, (cudaStream_t)stream);
     SL_CUDA(cudaGetLastError());
     return SL_OK;
 }
@@ -1106,8 +1104,7 @@ extern "C" sl_status sl_mesh_reset_t0(sl_mesh *m, void *stream)
 {
     if (!m) return fail(SL_E_ARG, "sl_mesh_reset_t0: mesh is NULL");
     m->t0_initial = true;
-    launch_reset_t0(m->d.t0_init, m->d.tv[0], m->d.tv[1], m->d.tv[2], m->d.t0, (int4 *)m->d.t0v, m->N,
-                    (cudaStream_t)stream);
+    launch_reset_t0(m->d.t0_init, (const int4 *)m->d.tri, (int4 *)m->d.t0v, m->N, (cudaStream_t)stream);
     SL_CUDA(cudaGetLastError());
     return SL_OK;
 }
@@ -1181,6 +1178,7 @@ extern "C" sl_status sl_mesh_reorder(sl_mesh *m, int32_t curve, int32_t *node_pe
     if (st != SL_OK) return st;
     if (m->stepped) {   // keep the walk state: bring the current T^0 back first
         SL_CUDA(cudaDeviceSynchronize());
+        launch_export_t0((const int4 *)m->d.t0v, m->d.t0, m->N, 0);
         SL_CUDA(cudaMemcpy(m->t0.data(), m->d.t0, sizeof(int32_t) * m->N, cudaMemcpyDeviceToHost));
     }
     st = reorder_host(m, curve, node_perm, tri_perm);
@@ -1229,7 +1227,11 @@ extern "C" sl_status sl_autotune_layout(sl_mesh *m, const sl_problem *probs, int
     SL_CUDA(cudaStreamSynchronize(s));
     std::vector<uint8_t> v0(esz * N), vl(esz * N);
     SL_CUDA(cudaMemcpy(v0.data(), v, esz * N, cudaMemcpyDeviceToHost));
-    if (m->stepped) SL_CUDA(cudaMemcpy(m->t0.data(), m->d.t0, sizeof(int32_t) * N, cudaMemcpyDeviceToHost));
+    if (m->stepped) {
+        launch_export_t0((const int4 *)m->d.t0v, m->d.t0, N, s);
+        SL_CUDA(cudaStreamSynchronize(s));
+        SL_CUDA(cudaMemcpy(m->t0.data(), m->d.t0, sizeof(int32_t) * N, cudaMemcpyDeviceToHost));
+    }
     // composite new -> old permutations (local) from the numbering at the call
     std::vector<int32_t> cn(N), ct(Nt), pn(N), pt(Nt);
     for (int32_t p = 0; p < m->n_problems; ++p) {
@@ -1386,7 +1388,7 @@ extern "C" sl_status sl_autotune(sl_mesh *m, const sl_problem *probs, int32_t pr
         SL_CUDA(cudaMalloc(&t_save, sizeof(int32_t) * m->N));
         SL_CUDA(cudaMalloc(&s_save, sizeof(unsigned long long) * kStatCounters));
         SL_CUDA(cudaMemcpy(v_save, v, vbytes, cudaMemcpyDeviceToDevice));
-        SL_CUDA(cudaMemcpy(t_save, m->d.t0, sizeof(int32_t) * m->N, cudaMemcpyDeviceToDevice));
+        launch_export_t0((const int4 *)m->d.t0v, (int32_t *)t_save, m->N, s);
         SL_CUDA(cudaMemcpy(s_save, m->d.stats, sizeof(unsigned long long) * kStatCounters, cudaMemcpyDeviceToDevice));
         SL_CUDA(cudaEventCreate(&e0));
         SL_CUDA(cudaEventCreate(&e1));
@@ -1496,8 +1498,7 @@ extern "C" sl_status sl_autotune(sl_mesh *m, const sl_problem *probs, int32_t pr
         }
         // restore values, T^0 and counters; keep the chosen configurations
         SL_CUDA(cudaMemcpyAsync(v, v_save, vbytes, cudaMemcpyDeviceToDevice, s));
-        SL_CUDA(cudaMemcpyAsync(m->d.t0, t_save, sizeof(int32_t) * m->N, cudaMemcpyDeviceToDevice, s));
-        launch_fill_t0v(m->d.t0, m->d.tv[0], m->d.tv[1], m->d.tv[2], (int4 *)m->d.t0v, m->N, s);
+        launch_fill_t0v((const int32_t *)t_save, m->d.tv[0], m->d.tv[1], m->d.tv[2], (int4 *)m->d.t0v, m->N, s);
         SL_CUDA(cudaMemcpyAsync(m->d.stats, s_save, sizeof(unsigned long long) * kStatCounters, cudaMemcpyDeviceToDevice, s));
         SL_CUDA(cudaMemsetAsync(m->d.status, 0, sizeof(uint32_t) * kStatusWords, s));
         SL_CUDA(cudaStreamSynchronize(s));

@@ -31,10 +31,10 @@ struct DeviceMesh {
     int32_t *tv[3] = {nullptr, nullptr, nullptr};   // vertex k of triangle j (global node index)
     int32_t *tn[3] = {nullptr, nullptr, nullptr};   // neighbour across edge opposite vertex k (global);
                                                     // boundary: -1 - side (0: x=0, 1: x=1, 2: y=0, 3: y=1)
-    int32_t *t0 = nullptr;            // start / last foot triangle of node i (global)
+    int32_t *t0 = nullptr;            // staging of T^0 as triangle indices (global) to and from the host
     int32_t *t0_init = nullptr;       // the initial start triangles (global)
     int32_t *pair_tri = nullptr;      // FP64: the triangle of each node's coordinate pair, or -1
-    void *t0v = nullptr;              // int4 (T^0, its vertex ids) per node
+    void *t0v = nullptr;              // T^0: int4 (3 T^0, its vertex ids) per node
     void *grid_t0v = nullptr;         // int4 start state per structured-grid triangle (strategy 2)
     int32_t *queue = nullptr;         // split steps: nodes left to the finish pass (N)
     uint32_t *queue_count = nullptr;

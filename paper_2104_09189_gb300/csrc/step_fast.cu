@@ -130,7 +130,7 @@ void launch_apply_df(const FastArgs &a, cudaStream_t s)
 // step's own path decides.  Once per mesh and numbering, for the full step's
 // foot_on_pair: with exact signs for every node of a step at which the field
 // vanishes, and for a third of a swirl's boundary nodes at every step, 20 steps
-// on 1.05 M nodes took 1.005 ms, 0.910 without; 1.18 M node-steps in two calls
+// on 1.05 M nodes took 1.005 ms, 0.910 without; two single steps on 296 k nodes
 // 70 -> 66 us.  (Asked in the lean pass instead it cost that pass 2 to 8 %.)
 __global__ void k_pair_tri(const __grid_constant__ FastArgs a, int32_t *__restrict__ pair_tri)
 {
@@ -306,17 +306,22 @@ __global__ void k_field_tables(FieldTableArgs a)
     }
 }
 
-// T^0 back to its initial triangles and the start-state cache with it, one
-// pass (sl_mesh_reset_t0).
-__global__ void k_reset_t0(const int32_t *__restrict__ t0_init, const int32_t *__restrict__ tv0,
-                           const int32_t *__restrict__ tv1, const int32_t *__restrict__ tv2, int32_t *__restrict__ t0,
-                           int4 *__restrict__ t0v, int64_t n)
+// T^0 back to its initial triangles (sl_mesh_reset_t0).
+__global__ void k_reset_t0(const int32_t *__restrict__ t0_init, const int4 *__restrict__ tri, int4 *__restrict__ t0v,
+                           int64_t n)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t j = t0_init[i];
-        t0[i] = j;
-        t0v[i] = make_int4(3 * j, tv0[j], tv1[j], tv2[j]);
-    }
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        t0v[i] = tri[t0_init[i]];
+}
+
+// T^0 as triangle indices.  The steps keep only the start states, 16 bytes per
+// node that moved; with the index beside them they wrote 20 (an FP32 swirl on 4.2 M
+// nodes 2.45 against 2.40 ms per 20 steps, a batch of 2.8 M 3.96 against 3.92 ms per
+// 50, 8 single steps on 491 k 174 against 170 us).
+__global__ void k_export_t0(const int4 *__restrict__ t0v, int32_t *__restrict__ t0, int64_t n)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        t0[i] = tri_of(t0v[i].x);
 }
 
 __global__ void k_fill_t0v(const int32_t *__restrict__ t0, const int32_t *__restrict__ tv0,
@@ -536,10 +541,14 @@ void launch_fill_t0v(const int32_t *t0, const int32_t *tv0, const int32_t *tv1, 
     if (n > 0) k_fill_t0v<<<grid_for(n, 256), 256, 0, s>>>(t0, tv0, tv1, tv2, t0v, n);
 }
 
-void launch_reset_t0(const int32_t *t0_init, const int32_t *tv0, const int32_t *tv1, const int32_t *tv2, int32_t *t0,
-                     int4 *t0v, int64_t n, cudaStream_t s)
+void launch_reset_t0(const int32_t *t0_init, const int4 *tri, int4 *t0v, int64_t n, cudaStream_t s)
 {
-    if (n > 0) k_reset_t0<<<grid_for(n, 256), 256, 0, s>>>(t0_init, tv0, tv1, tv2, t0, t0v, n);
+    if (n > 0) k_reset_t0<<<grid_for(n, 256), 256, 0, s>>>(t0_init, tri, t0v, n);
+}
+
+void launch_export_t0(const int4 *t0v, int32_t *t0, int64_t n, cudaStream_t s)
+{
+    if (n > 0) k_export_t0<<<grid_for(n, 256), 256, 0, s>>>(t0v, t0, n);
 }
 
 void launch_field_tables(const FieldTableArgs &a, cudaStream_t s)

@@ -63,9 +63,7 @@ struct FastArgs {
     const int32_t *t0_init;       // the node's initial incident triangle
     const int32_t *pair_tri;      // FP64 meshes: the triangle that holds the node's coordinate pair (not its
                                   // double coordinates), or -1 when there are several
-    int32_t *t0;
-    int4 *t0v;                    // per node: (3 T^0, T[0][T^0], T[1][T^0], T[2][T^0]), kept in
-                                  // step with t0
+    int4 *t0v;                    // T^0 per node (in place): (3 T^0, T[0][T^0], T[1][T^0], T[2][T^0])
     const void *vin;              // FP64: float2 (hi, lo) values, or the doubles (io); FP32: float values
     void *vout;
     int32_t io;                   // FP64: kIoIn: vin holds doubles; kIoOut: vout takes doubles.  Not in the
@@ -290,8 +288,9 @@ void launch_pair_tri(const FastArgs &a, int32_t *pair_tri, cudaStream_t s);
 // t0v[i] = (3 t0[i], its three vertex ids in slot order)
 void launch_fill_t0v(const int32_t *t0, const int32_t *tv0, const int32_t *tv1, const int32_t *tv2, int4 *t0v,
                      int64_t n, cudaStream_t s);
-// t0 = t0_init and the start-state cache with it, one pass
-void launch_reset_t0(const int32_t *t0_init, const int32_t *tv0, const int32_t *tv1, const int32_t *tv2, int32_t *t0,
-                     int4 *t0v, int64_t n, cudaStream_t s);
+// the same from the triangles' start states (FastArgs::tri): T^0 back to the initial triangles
+void launch_reset_t0(const int32_t *t0_init, const int4 *tri, int4 *t0v, int64_t n, cudaStream_t s);
+// t0[i] = the triangle of t0v[i]
+void launch_export_t0(const int4 *t0v, int32_t *t0, int64_t n, cudaStream_t s);
 
 }  // namespace sl

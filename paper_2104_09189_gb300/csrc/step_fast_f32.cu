@@ -169,7 +169,6 @@ __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int 
         excluded = true;
         if (a.parent) {
             // strategy (c): the children start where this node would have
-            a.t0[i] = a.t0[a.parent[i]];
             a.t0v[i] = a.t0v[a.parent[i]];
         }
         if (kDebug) {
@@ -411,7 +410,6 @@ __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int 
         ((float *)a.vout)[i] = interpolate_f32(th1, th2, v1, v2, v3);
         if (!kCount && (P.flags & kFastEmit)) emit_weights_f32(a, i, w0, w1, w2, th1, th2);
         if ((moved || (kExt && a.parent)) && !(kExt && a.keep_t0)) {
-            a.t0[i] = j;
             a.t0v[i] = make_int4(3 * j, w0, w1, w2);
         }
         if (c.limit_cnt) atomicOr(a.status, 1u << SL_E_WALK_LIMIT);
@@ -611,7 +609,6 @@ __device__ __forceinline__ bool lean_node_f32(const FastArgs &a, int64_t i, int 
     ((float *)a.vout)[i] = interpolate_f32(th1, th2, v1, v2, v3);
     if (P.flags & kFastEmit) emit_weights_f32(a, i, tq.y, tq.z, tq.w, th1, th2);
     if (moved && !(kExt && a.keep_t0)) {
-        a.t0[i] = tri_of_f32(tq.x);
         a.t0v[i] = tq;
     }
     return true;

@@ -906,7 +906,6 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
             c.excluded = 1;
             if (a.parent) {
                 // strategy (c): the children start where this node would have
-                a.t0[i] = a.t0[a.parent[i]];
                 a.t0v[i] = a.t0v[a.parent[i]];
             }
             if (kDebug) {
@@ -942,16 +941,12 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     // coordinate, so without this the exact stage would run on a
     // rounding-sized offset every step.
     if (at_node && (tq.y == (int32_t)i || tq.z == (int32_t)i || tq.w == (int32_t)i)) {
-        const int32_t j0 = tri_of(tq.x);
         keep_value(a, i);
         if (!kCount && (P.flags & kFastEmit)) emit_own(a, i);
-        if (kExt && a.parent && !a.keep_t0) {
-            a.t0[i] = j0;
-            a.t0v[i] = tq;
-        }
+        if (kExt && a.parent && !a.keep_t0) a.t0v[i] = tq;
         if (kDebug) {
             write_node_foot(a, i);
-            if (a.dbg.tri) a.dbg.tri[i] = j0;
+            if (a.dbg.tri) a.dbg.tri[i] = tri_of(tq.x);
             if (a.dbg.moves) a.dbg.moves[i] = 0;
             if (a.dbg.flags) a.dbg.flags[i] = (uint8_t)(flags | SL_NODE_DEGENERATE);
         }
@@ -1159,10 +1154,8 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
         if (at_node && (w0 == (int)i || w1 == (int)i || w2 == (int)i)) emit_own(a, i);
         else emit_weights(a, i, w0, w1, w2, n1, n2, den, flags & SL_NODE_CLIPPED);
     }
-    if ((hops > 0 || (kExt && a.parent)) && !(kExt && a.keep_t0)) {
-        a.t0[i] = j;
+    if ((hops > 0 || (kExt && a.parent)) && !(kExt && a.keep_t0))
         a.t0v[i] = make_int4(3 * j, w0, w1, w2);
-    }
     if (c.limit) atomicOr(a.status, 1u << SL_E_WALK_LIMIT);
     if (flags & SL_NODE_RANGE) atomicOr(a.status, 1u << SL_E_ARG);
     if (kDebug) {

@@ -13,8 +13,7 @@ struct StepArgs {
     const void *xy;               // double2[N] or float2[N]
     const int32_t *tv[3];         // triangle vertices (global node indices), SoA
     const int32_t *tn[3];         // neighbours (global triangle indices, -1 = boundary), SoA
-    int32_t *t0;                  // start / located triangle per node (in place)
-    int4 *t0v;                    // (T^0, its vertex ids) per node, kept in step with t0
+    int4 *t0v;                    // start / located triangle per node (in place): (3 T^0, its vertex ids)
     const void *vin;              // V^n
     void *vout;                   // V^{n+1}
     const ProbStep *probs;        // per-problem data of this step (device)

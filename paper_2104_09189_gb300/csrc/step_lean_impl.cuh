@@ -192,10 +192,7 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
         val = p1_value_of(V1, V2, V3, t.n1, t.n2, t.den);
     put_value(a, i, val);
     if (P.flags & kFastEmit) emit_weights(a, i, tq.y, tq.z, tq.w, t.n1, t.n2, t.den, clipped);
-    if (moved && !(kExt && a.keep_t0)) {
-        a.t0[i] = tri_of(tq.x);
-        a.t0v[i] = tq;
-    }
+    if (moved && !(kExt && a.keep_t0)) a.t0v[i] = tq;
     return true;
 }
 

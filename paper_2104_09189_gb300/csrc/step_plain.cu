@@ -98,10 +98,7 @@ __device__ __forceinline__ void plain_walk_value(const StepArgs &a, int64_t i, i
     const int ia = a.tv[0][j], ib = a.tv[1][j], ic = a.tv[2][j];
     const double v = __dadd_rn(__dadd_rn(__dmul_rn(th1, vin[ia]), __dmul_rn(th2, vin[ib])), __dmul_rn(th3, vin[ic]));
     ((double *)a.vout)[i] = v;
-    if (!(kExt && a.keep_t0)) {
-        a.t0[i] = j;
-        a.t0v[i] = make_int4(3 * j, ia, ib, ic);     // the start state of the fast kernels
-    }
+    if (!(kExt && a.keep_t0)) a.t0v[i] = make_int4(3 * j, ia, ib, ic);
     if (limit_cnt) atomicOr(a.status, 1u << SL_E_WALK_LIMIT);
     if (flags & SL_NODE_RANGE) atomicOr(a.status, 1u << SL_E_ARG);
     if (kDebug) {
@@ -137,7 +134,7 @@ __global__ void __launch_bounds__(256) k_step_plain_f64(StepArgs a)
         if (!kExt) {
             double X, Y;
             const bool clipped = foot_clip_f64(xi.x, xi.y, P.dt, fx, fy, X, Y);
-            plain_walk_value<kDebug, false>(a, i, a.t0[i], X, Y, clipped, hops, exact_tests, clipped_cnt,
+            plain_walk_value<kDebug, false>(a, i, a.t0v[i].x / 3, X, Y, clipped, hops, exact_tests, clipped_cnt,
                                             fallback_cnt, limit_cnt);
         } else {
             const double qx = __dsub_rn(xi.x, __dmul_rn(P.dt, fx)), qy = __dsub_rn(xi.y, __dmul_rn(P.dt, fy));
@@ -148,7 +145,6 @@ __global__ void __launch_bounds__(256) k_step_plain_f64(StepArgs a)
                 excluded_cnt = 1;
                 if (a.parent) {
                     // strategy (c): the children start where this node would have
-                    a.t0[i] = a.t0[a.parent[i]];
                     a.t0v[i] = a.t0v[a.parent[i]];
                 }
                 if (kDebug) {
@@ -168,7 +164,7 @@ __global__ void __launch_bounds__(256) k_step_plain_f64(StepArgs a)
                 double X, Y;
                 const bool clipped = clip_to_square(xi.x, xi.y, qx, qy, X, Y);
                 const int32_t j0 = a.grid_M > 0 ? a.grid_t0v[grid_slot((float)X, (float)Y, a.grid_M)].x / 3
-                                                : a.t0[a.parent ? (int64_t)a.parent[i] : i];
+                                                : a.t0v[a.parent ? (int64_t)a.parent[i] : i].x / 3;
                 plain_walk_value<kDebug, true>(a, i, j0, X, Y, clipped, hops, exact_tests, clipped_cnt,
                                                fallback_cnt, limit_cnt);
             }
