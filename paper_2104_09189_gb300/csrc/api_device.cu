@@ -475,7 +475,7 @@ FastArgs make_fast_args(const sl_mesh *m, const FastProb *fp, const void *vin, v
     a.chunk_prob = (const int2 *)m->d.chunk_prob;
     a.nprob = m->n_problems;
     a.walk_cap = m->opt_walk_cap > 0 ? m->opt_walk_cap : default_walk_cap(m);
-    a.capped = m->opt_walk_cap > 0;
+    a.lean_moves = m->opt_walk_cap > 0 ? 0 : 8;
     a.N = m->N;
     a.status = m->d.status;
     a.stats = m->d.stats;

@@ -83,7 +83,8 @@ struct FastArgs {
                                   // problem (chunk_problem); else NULL
     int32_t nprob;
     int32_t walk_cap;
-    int32_t capped;               // host side: walk_cap is the caller's (the full node step keeps to it)
+    int32_t lean_moves;           // FP64: certified moves a lean pass may add to its hops (8; 0 under a
+                                  // hop cap of the caller's, which the hops alone keep to)
     int64_t N;
     uint32_t *status;
     unsigned long long *stats;
@@ -191,7 +192,7 @@ void launch_lean_df_c3(const FastArgs &a, cudaStream_t s);
 void launch_lean_df_c4(const FastArgs &a, cudaStream_t s);
 void launch_lean_df_c5(const FastArgs &a, cudaStream_t s);
 void launch_lean_df_ext(const FastArgs &a, cudaStream_t s);
-// the full node step alone: statistics, debug outputs, strategy (c), a hop cap
+// the full node step alone: statistics, debug outputs, strategy (c)
 void launch_full_df(const FastArgs &a, bool stats, bool debug, cudaStream_t s);
 // the two passes of a split step: lean settle pass, then the finish pass over
 // its queue (reset: zero the queue counter first)

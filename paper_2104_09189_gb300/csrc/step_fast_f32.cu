@@ -148,14 +148,15 @@ struct CountersF32 {
 // strategies (a), (c) and the direct structured-grid start); the default
 // variant compiles them out.
 // kCount: the variants that count or report (statistics, debug outputs).
-template <bool kDebug, bool kCount, bool kExt>
+// kInts: exact signs in integers first, for the nodes a lean pass leaves, which
+// a whole step waits for.  Off in the kernel of this step alone: the levels of
+// strategy (c), a few hundred launches of a few hundred nodes per step, are bound by
+// launch and code fetch, and the larger loop body cost 8 % of a run (20 steps
+// on 149 k nodes 32.4 -> 35.1 ms; 30.4 without it).
+template <bool kDebug, bool kCount, bool kExt, bool kInts>
 __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int pi, CountersF32 &c)
 {
     const FastProb &P = a.single ? a.prob0 : a.probs[pi];
-    if (!kCount && (P.flags & kFastUse)) {
-        apply_weights_f32(a, i);
-        return;
-    }
     const float2 xf = a.xyf[i];
     float X, Y;
     foot_f32(P, a, i, xf.x, xf.y, X, Y);
@@ -267,9 +268,9 @@ __device__ __forceinline__ void step_node_f32(const FastArgs &a, int64_t i, int 
                 // conversions of the loop-invariant foot inside it
                 const int32_t jj = tri_of_f32(e0), sa = e0 - 3 * jj, sb = e1 - 3 * jj, sc = 3 - sa - sb;
                 const float2 A = a.xyf[a.tv[sa][jj]], B = a.xyf[a.tv[sb][jj]], C = a.xyf[a.tv[sc][jj]];
-                if (!kCount) {
-                    // integers where the coordinates allow (the counting variants
-                    // take the stages below, which give the same signs)
+                if (kInts) {
+                    // integers where the coordinates allow (the stages below give
+                    // the same signs)
                     long long ax, ay, bx, by, cx, cy, x, y;
                     if (slp::fixed62(A.x, ax) & slp::fixed62(A.y, ay) & slp::fixed62(B.x, bx) &
                         slp::fixed62(B.y, by) & slp::fixed62(C.x, cx) & slp::fixed62(C.y, cy) & slp::fixed62(X, x) &
@@ -442,7 +443,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_step_fast_f32(const __gr
                    : (kExt && a.order ? problem_of(a.node_off, a.nprob, i) : chunk_problem(a.chunk_prob, a.node_off, i));
     pdl_launch_dependents();
     pdl_wait();
-    if (active) step_node_f32<kDebug, kStats || kDebug, kExt>(a, i, pi, c);
+    if (active) step_node_f32<kDebug, kStats || kDebug, kExt, false>(a, i, pi, c);
     if (kStats)
         warp_stats(a.stats, active, c.hops, c.exact_tests, c.clipped_cnt, c.fallback_cnt, c.limit_cnt, c.fp64_tests,
                    c.excluded_cnt);
@@ -624,7 +625,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_lean_f32(const __grid_co
     const int pi = kSingle || a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i);
     if (lean_node_f32<kExt, kSingle>(a, i, pi)) return;
     CountersF32 c;
-    step_node_f32<false, false, kExt>(a, i, pi, c);
+    step_node_f32<false, false, kExt, true>(a, i, pi, c);
 }
 
 template <int kBlock, int kMinBlocks, bool kExt = false>
@@ -646,18 +647,22 @@ static void launch_f32_cfg(const FastArgs &a, bool stats, bool debug, cudaStream
         else launch_step_kernel(k_step_fast_f32<true, false, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
     } else {
         if (debug) launch_step_kernel(k_step_fast_f32<false, true, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
-        else if constexpr (kExt)    // strategy (c), a hop cap; the lean kernel takes the others
+        else if constexpr (kExt)    // strategy (c); the lean kernel takes the others
             launch_step_kernel(k_step_fast_f32<false, false, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
     }
 }
 
 void launch_fast_f32(const FastArgs &a, bool stats, bool debug, int config, cudaStream_t s)
 {
-    // statistics, debug outputs, a hop cap of the caller's and strategy (c): the
-    // full node step, one configuration (128 x 8)
+    // statistics, debug outputs and strategy (c): the full node step, one
+    // configuration (128 x 8).  A hop cap of the caller's needs no route of its
+    // own: a lean walk makes the full step's hops one by one and hands a node that
+    // reaches the cap outside its triangle to the full step (no jump table then; a
+    // 2048^2-node swirl of 20 steps under a cap it never meets: 6.31 ms in the full
+    // step, 4.40 here)
     const bool ext = a.exclude || a.order || a.grid_M > 0 || a.keep_t0;
-    if (stats || debug || a.order || a.capped) {
-        if (ext || !(stats || debug)) launch_f32_cfg<128, 8, true>(a, stats, debug, s);
+    if (stats || debug || a.order) {
+        if (ext) launch_f32_cfg<128, 8, true>(a, stats, debug, s);
         else launch_f32_cfg<128, 8>(a, stats, debug, s);
         return;
     }

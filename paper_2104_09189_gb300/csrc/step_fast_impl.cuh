@@ -869,15 +869,17 @@ struct NodeCounters {
 // (T[0][j], T[1][j], T[2][j]), so the result depends on the located triangle
 // and the foot only, not on the path of the walk.
 //
-// kCount: the variants that count or report (statistics, debug outputs).
-template <bool kDebug, bool kCount, bool kExt, bool kCompact>
+// kLean: the nodes a lean (or settle) pass leaves, where nothing is counted: a
+// whole step waits for them, so exact signs are taken in integers first and a
+// foot on its node's pair takes its known triangle.  Off where the step counts
+// or reports, and in the kernel of this step alone: the levels of strategy (c),
+// a few hundred launches of a few hundred nodes per step, are bound by launch and
+// code fetch, and the code they hardly ever run cost 5 % (20 steps on 149 k nodes
+// 37.8 -> 35.8 ms without it).
+template <bool kDebug, bool kLean, bool kExt, bool kCompact>
 __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, NodeCounters &c)
 {
     const FastProb &P = a.single ? a.prob0 : a.probs[pi];
-    if (!kCount && (P.flags & kFastUse)) {
-        put_value(a, i, apply_weights(a, i));
-        return;
-    }
     const float4 xq = a.xyq[i];
     const df x = df_make(xq.x, xq.z), y = df_make(xq.y, xq.w);
     df DX, DY;
@@ -942,7 +944,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     // rounding-sized offset every step.
     if (at_node && (tq.y == (int32_t)i || tq.z == (int32_t)i || tq.w == (int32_t)i)) {
         keep_value(a, i);
-        if (!kCount && (P.flags & kFastEmit)) emit_own(a, i);
+        if (kLean && (P.flags & kFastEmit)) emit_own(a, i);
         if (kExt && a.parent && !a.keep_t0) a.t0v[i] = tq;
         if (kDebug) {
             write_node_foot(a, i);
@@ -957,8 +959,8 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     int w0 = tq.y, w1 = tq.z, w2 = tq.w;
     // A foot that ends as its node's coordinate pair, within rounding of the
     // node, is a point of the mesh alone, and its triangle is known (k_pair_tri;
-    // the counting variants walk there).
-    const int32_t known = !kCount && foot_on_pair(a.xyq[i], X, Y) ? a.pair_tri[i] : -1;
+    // without kLean it is walked to).
+    const int32_t known = kLean && foot_on_pair(a.xyq[i], X, Y) ? a.pair_tri[i] : -1;
     bool ids = true;           // w0..w2 are the vertex ids of the current triangle
     const uint32_t cap = (uint32_t)a.walk_cap;
     uint32_t &hops = c.hops;
@@ -1068,7 +1070,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
         }
         if (s1 == 2 || s2 == 2 || s3 == 2) {
             // exact signs on the double coordinates and the exact foot
-            const uint32_t r = exact_signs<kCount>(a.xyd, w0, w1, w2, X, Y, (s1 == 2 ? 1u : 0u) | (s2 == 2 ? 2u : 0u) | (s3 == 2 ? 4u : 0u));
+            const uint32_t r = exact_signs<!kLean>(a.xyd, w0, w1, w2, X, Y, (s1 == 2 ? 1u : 0u) | (s2 == 2 ? 2u : 0u) | (s3 == 2 ? 4u : 0u));
             if (s1 == 2) s1 = unpack_sign(r, 0);
             if (s2 == 2) s2 = unpack_sign(r, 1);
             if (s3 == 2) s3 = unpack_sign(r, 2);
@@ -1150,7 +1152,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
             put_value(a, i, p1_value_of(V1, V2, V3, n1, n2, den));
         }
     }
-    if (!kCount && (P.flags & kFastEmit)) {
+    if (kLean && (P.flags & kFastEmit)) {
         if (at_node && (w0 == (int)i || w1 == (int)i || w2 == (int)i)) emit_own(a, i);
         else emit_weights(a, i, w0, w1, w2, n1, n2, den, flags & SL_NODE_CLIPPED);
     }
@@ -1181,7 +1183,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_step_fast_df(const __gri
     // level (a level mixes problems)
     const int pi = !active || a.nprob == 1 ? 0
                    : (kExt && a.order ? problem_of(a.node_off, a.nprob, i) : chunk_problem(a.chunk_prob, a.node_off, i));
-    if (active) step_node<kDebug, kStats || kDebug, kExt, kCompact>(a, i, pi, c);
+    if (active) step_node<kDebug, false, kExt, kCompact>(a, i, pi, c);
     if (kStats) warp_stats(a.stats, active, c.hops, c.exact, c.clipped, c.fallback, c.limit, c.filter2, c.excluded);
 }
 
@@ -1331,7 +1333,7 @@ __global__ void __launch_bounds__(128, 8) k_finish_df(const __grid_constant__ Fa
     for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < count; q += gridDim.x * blockDim.x) {
         NodeCounters c;
         const int64_t i = a.queue[q];
-        step_node<kDebug, kStats || kDebug, false, kCompact>(a, i, a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i), c);
+        step_node<kDebug, !(kStats || kDebug), false, kCompact>(a, i, a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i), c);
         tot.hops += c.hops;
         hmax = c.hops > hmax ? c.hops : hmax;
         tot.exact += c.exact;

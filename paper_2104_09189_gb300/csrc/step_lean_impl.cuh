@@ -171,7 +171,7 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
         // between triangles the path decides: step_node's, as long as the FP32
         // walk from T^0 ended here
         if (d == kIn || (d == kInShared && !jumped && n == 0)) break;
-        if (d >= kIn || n == 8) return false;
+        if (d >= kIn || n == a.lean_moves) return false;
         const int32_t u = a.tn[d][tri_of(tq.x)];
         if (u < 0) return false;
         tq = __ldg(&a.tri[u]);
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocks) k_lean_df(const __grid_con
     const int pi = kSingle || a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i);
     if (lean_node<kExt, kCompact, kSingle>(a, i, pi)) return;
     NodeCounters c;
-    step_node<false, false, kExt, kCompact>(a, i, pi, c);
+    step_node<false, true, kExt, kCompact>(a, i, pi, c);
 }
 
 template <int kBlock, int kMinBlocks, bool kExt = false>

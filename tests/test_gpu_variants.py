@@ -138,6 +138,42 @@ def test_a_hop_cap_holds_without_counting(precision):
             assert e.value.status == sl.SL_E_WALK_LIMIT
 
 
+@pytest.mark.parametrize("precision,records", [(sl.SL_FP64, 0), (sl.SL_FP64, 1), (sl.SL_FP32, 0)],
+                         ids=["fp64", "fp64-records8", "fp32"])
+def test_every_hop_cap_is_the_plain_step(precision, records):
+    """Caps around the lengths of the walks: the same outcome with and without
+    the counting variant, and where no walk gave up the same triangles and values
+    (the fallback's choices depend on the node and the hop alone)."""
+    m = si.grid_mesh(60, 0.25, 7)
+    f = si.swirl_field()
+    g = DeviceRun(m, f, 0.05, precision=precision)
+    sl.sl_mesh_set_option(g.h, sl.SL_OPT_RECORDS, records)
+    t = g.torch
+    v = g.to_dev(si.cosine_bump(m.xy))
+    outcomes = set()
+    for cap in range(1, 13):
+        sl.sl_mesh_set_option(g.h, sl.SL_OPT_WALK_CAP, cap)
+        got = []
+        for debug in (True, False):
+            sl.sl_mesh_reset_t0(g.h)
+            w = t.empty_like(v)
+            moves = t.zeros(m.n_nodes, dtype=t.int32, device=g.dev)
+            sl.sl_step(g.h, g.probs, 1, v, w, debug={"moves": moves} if debug else None)
+            try:
+                sl.sl_mesh_status(g.h)
+                status = sl.SL_OK
+            except sl.SLError as e:
+                status = e.status
+            j = t.empty(m.n_nodes, dtype=t.int32, device=g.dev)
+            sl.sl_mesh_get_t0(g.h, j)
+            got.append((status, w, j))
+        assert got[0][0] == got[1][0], f"cap {cap}"
+        outcomes.add(got[0][0])
+        if got[0][0] == sl.SL_OK:
+            assert bool((got[0][1] == got[1][1]).all()) and bool((got[0][2] == got[1][2]).all()), f"cap {cap}"
+    assert outcomes == {sl.SL_OK, sl.SL_E_WALK_LIMIT}
+
+
 def test_jump_table_of_uneven_batch():
     """Meshes of 9 to 10 000 nodes in one batch, each with a table of its own."""
     import torch
