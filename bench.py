@@ -4,7 +4,7 @@
 One benchmark step is one run of the whole hot path over the workload: the
 S-step time loop of Algorithm 2 (foot, clip, walk from the previous foot
 triangle, P1) replayed as one CUDA graph, starting from the initial start
-triangles (so the first step's long strategy-(a) walk is included).
+triangles (so the first step's long way from them is included).
 
 Default workload: the 4096 x 4096 graded, jittered mesh (16 785 409 nodes,
 33 554 432 triangles), solid rotation, Gaussian data, dt = 0.02, 50 steps,
@@ -35,6 +35,9 @@ if ROOT not in sys.path:
 import sl_inputs as si  # noqa: E402
 
 BYTES_PER_NODE = {"fp64": 64, "fp32": 48}   # algorithmic bytes per node-update
+# ... of a steady field: the first step also stores the weights (ids, theta, a
+# bound), the later ones read them, V^n and write V^{n+1}
+STEADY_BYTES = {"fp64": (96, 48), "fp32": (68, 28)}
 
 
 def parse():
@@ -104,11 +107,46 @@ def whole_job_value(nodes_per_rank, steps_per_run, runs, world, seconds):
     return nodes_per_rank * steps_per_run * runs * world / seconds
 
 
+def is_steady(prob_list, steps_per_run):
+    """A run the library steps with the weights of its first step: 4 steps and
+    more of fields that do not depend on time."""
+    return steps_per_run >= 4 and all(
+        p.field.kind in (si.FIELD_ZERO, si.FIELD_ROTATION) or
+        (p.field.kind == si.FIELD_AFFINE and p.field.packed()[3] == 0 and p.field.packed()[7] == 0) for p in prob_list)
+
+
+def run_bytes_per_node(prob_list, precision, steps):
+    """Algorithmic bytes per node-update of a run of `steps` steps: the steady
+    problems of the list move fewer in the steps after their first one."""
+    total = 0.0
+    for p in prob_list:
+        if is_steady([p], steps):
+            first, later = STEADY_BYTES[precision]
+            total += p.mesh.n_nodes * (first + (steps - 1) * later) / steps
+        else:
+            total += p.mesh.n_nodes * BYTES_PER_NODE[precision]
+    return total / sum(p.mesh.n_nodes for p in prob_list)
+
+
 def launches_per_run(steps_per_run, double_float):
-    """Kernels one timed run launches: the start-cache fill after the T^0
-    reset, one step kernel per step and, for the double-float path, the value
-    conversions to and from (hi, lo) pairs."""
+    """Kernels of a run with nothing folded: the T^0 reset, one step kernel
+    per step and, for the double-float path, the value conversions to and from
+    (hi, lo) pairs."""
     return steps_per_run + 1 + (2 if double_float else 0)
+
+
+def run_launches(steps_per_run, double_float, split, steady):
+    """Kernels one timed run launches.  The first and the last step read and
+    write the caller's doubles themselves, so the conversions are left out,
+    except that a split step takes pairs only and that an odd number of steps
+    leaves one of them on the wrong buffer (one conversion either way); every
+    split step (never the first, none in a steady run) has a finish pass."""
+    n = launches_per_run(steps_per_run, double_float)
+    if double_float:
+        split = split and not steady
+        n -= 1 if split or steps_per_run % 2 else 2
+        n += steps_per_run - 1 if split else 0
+    return n
 
 
 class ClockSampler:
@@ -195,18 +233,17 @@ def build_workload(args):
     return Workload(prob.name, [prob], prob.precision, prob.n_steps, desc)
 
 
-TRAFFIC_SOURCES = ("step_fast.cu", "step_fast_impl.cuh", "step_fast_c01.cu", "step_fast_c23.cu", "step_fast_c45.cu", "step_fast.cuh", "df.cuh", "predicates.cuh", "step_common.cuh", "step_kernels.cuh")
+TRAFFIC_SOURCES = ("step_fast.cu", "step_fast_impl.cuh", "step_lean_impl.cuh", "step_fast_c01.cu", "step_fast_c23.cu", "step_fast_c45.cu", "step_fast.cuh", "df.cuh", "predicates.cuh", "step_common.cuh", "step_kernels.cuh")
 
 
-def committed_traffic(workload_key, split=0):
-    """DRAM bytes per step of the dominant kernel (the fused step kernel, or
-    the settle + finish passes of a split step) from the committed ncu
-    summary (profiles/k_step_fast_df_c3_traffic.md), or None when the kernel
-    sources changed since that capture, the workload differs or the form was
-    not captured."""
+def committed_traffic(workload_key):
+    """DRAM bytes per step of a run (the first step in the fused kernel, the
+    later ones applying its weights) from the committed ncu summary
+    (profiles/k_apply_df_c3_traffic.md), or None when the kernel sources
+    changed since that capture or the workload differs."""
     import hashlib
     here = os.path.dirname(os.path.abspath(__file__))
-    path = os.path.join(here, "profiles", "k_step_fast_df_c3_traffic.md")
+    path = os.path.join(here, "profiles", "k_apply_df_c3_traffic.md")
     if not os.path.exists(path):
         return None
     fields = {}
@@ -219,7 +256,7 @@ def committed_traffic(workload_key, split=0):
         h.update(open(os.path.join(here, "paper_2104_09189_gb300", "csrc", f), "rb").read())
     if fields.get("source_sha256") != h.hexdigest() or fields.get("workload") != workload_key:
         return None
-    key = "traffic_bytes_per_step_split" if split else "traffic_bytes_per_step_fused"
+    key = "traffic_bytes_per_step"
     return float(fields[key]) if key in fields else None
 
 
@@ -384,7 +421,7 @@ def secondary_workload(sl, torch, config, precision, runs, warmup, oracle_cache)
         oracle_cache[key] = (oracle_reference(wl.probs, S), time.perf_counter() - t0)
     want, oracle_s = oracle_cache[key]
     err = error_vs_oracle(wl.probs, got, want)
-    bpn = BYTES_PER_NODE[precision]
+    bpn = run_bytes_per_node(wl.probs, precision, S)
     peaks, peak_src = measured_peaks()
     value = N * S / (ms / 1e3)
     achieved = bpn * N * S / (ms / 1e3) / 1e9
@@ -489,8 +526,11 @@ def run_study(args):
                 sl.sl_mesh_set_option(h, sl.SL_OPT_STRATEGY, strategy)
                 sl.sl_mesh_stats(h, reset=True)
                 v.copy_(v0)
-                sl.sl_run(h, probs, 0, S, v, w, use_graph=True)       # records the graph; statistics
+                sl.sl_run(h, probs, 0, S, v, w, use_graph=True)       # statistics
                 st = sl.sl_mesh_stats(h, reset=True)
+                if strategy != 3:
+                    sl.sl_mesh_reset_t0(h)
+                    sl.sl_run(h, probs, 0, S, v, w, use_graph=True)   # records the graph
                 sl.sl_mesh_reset_t0(h)
                 v.copy_(v0)
                 torch.cuda.synchronize()
@@ -515,14 +555,16 @@ def run_study(args):
 
 
 def _timed_run(sl, torch, h, probs, S, v, v0, w):
-    """One S-step run (graph) for the statistics, then the same run timed
-    with CUDA events.  Returns (ms, stats of the first run)."""
+    """One S-step run for the statistics, the same run again to record its graph,
+    then a replay timed with CUDA events.  Returns (ms, stats of the first run)."""
     stream = torch.cuda.current_stream()
     sl.sl_mesh_stats(h, reset=True)
     sl.sl_mesh_reset_t0(h)
     v.copy_(v0)
     sl.sl_run(h, probs, 0, S, v, w, use_graph=True)
     st = sl.sl_mesh_stats(h, reset=True)
+    sl.sl_mesh_reset_t0(h)
+    sl.sl_run(h, probs, 0, S, v, w, use_graph=True)
     sl.sl_mesh_reset_t0(h)
     v.copy_(v0)
     torch.cuda.synchronize()
@@ -646,6 +688,7 @@ def main():
     if not args.pdl:
         sl.sl_mesh_set_option(h, sl.SL_OPT_PDL, 0)
     split = (args.split if args.split is not None else (tune or {}).get("split", 0)) if prec == sl.SL_FP64 else 0
+    steady = is_steady(wl.probs, S) and args.kernel != 1
     setup_s = time.perf_counter() - t_setup
 
     def one_run():
@@ -712,9 +755,10 @@ def main():
               "note": "eager launches, one run, after the timed region"}
 
     # the effective gather roofline of a later step: a kernel making exactly
-    # its memory accesses (on the current start triangles) with no arithmetic
+    # its memory accesses (on the current start triangles) with no arithmetic;
+    # not for a steady run, whose later steps gather no vertices
     gather = None
-    if prec == sl.SL_FP64 and args.kernel != 1:
+    if prec == sl.SL_FP64 and args.kernel != 1 and not steady:
         probe_ms = sl.sl_probe_gather(h, v, w, reps=20)
         gather = {"probe_ms": probe_ms, "later_step_ms": rest_ms, "frac_of_gather_bound": probe_ms / rest_ms,
                   "kernel": "k_gather_probe (node pair and start state, three vertex pairs, three values, one write)"}
@@ -741,18 +785,20 @@ def main():
 
     value = whole_job_value(N, S, args.steps, world, elapsed)
     launch_s = elapsed / (args.steps * S)
-    bpn = BYTES_PER_NODE[wl.precision]
+    bpn = BYTES_PER_NODE[wl.precision] if args.kernel == 1 else run_bytes_per_node(wl.probs, wl.precision, S)
     peaks, peak_src = measured_peaks()
     achieved_gbs = bpn * N / launch_s / 1e9
     hbm = peaks.get("hbm_gbs", 6800.0)
 
-    def phase(ms):
-        a = bpn * N / (ms / 1e3) / 1e9
+    def phase(ms, steps):
+        b = BYTES_PER_NODE[wl.precision] if args.kernel == 1 else run_bytes_per_node(wl.probs, wl.precision, steps)
+        a = b * N / (ms / 1e3) / 1e9
         return {"ms": ms, "achieved": a, "frac": a / hbm}
 
-    phase_roofline = {"first_step": phase(first_ms), "later_steps": phase(rest_ms),
-                      "note": "eager launches after the timed region; the first step walks from the initial "
-                              "incident triangles, the later ones from the previous foot triangles"}
+    phase_roofline = {"first_step": phase(first_ms, 1), "later_steps": phase(rest_ms, S - 1),
+                      "note": "eager launches after the timed region, each phase a run of its own; the first step "
+                              "starts far from its feet, the later ones locate from the previous foot triangles once "
+                              "and, in a steady run, apply the weights they found"}
 
     # end to end through the C ABI with host buffers (pinned)
     e2e = None
@@ -813,20 +859,22 @@ def main():
         "config": workload_config(args, wl),
         "roofline": {"bound": "hbm", "achieved": achieved_gbs, "peak": peaks.get("hbm_gbs", 6800.0),
                      "unit": "GB/s", "frac": achieved_gbs / peaks.get("hbm_gbs", 6800.0),
-                     "traffic": (committed_traffic(f"{args.config} {wl.precision}", split)
+                     "traffic": (committed_traffic(f"{args.config} {wl.precision}")
                                  if args.kernel != 1 and args.cells is None else None),
                      "peak_source": peak_src,
                      "algorithmic_bytes_per_node": bpn,
                      "kernel": ("k_step_plain_f64" if args.kernel == 1 else
-                                ("k_step_fast_df" + (" (later steps split: k_settle_df + k_finish_df)" if split else "")
-                                 if prec == sl.SL_FP64 else "k_step_fast_f32"))
+                                ("k_lean_df" + (" (later steps: k_apply_df)" if steady else
+                                                " (later steps split: k_settle_df + k_finish_df)" if split else "")
+                                 if prec == sl.SL_FP64 else
+                                 "k_lean_f32" + (" (later steps: k_apply_f32)" if steady else "")))
                                + " (one step over all nodes; duration = timed region / steps)",
                      "launch_ms": launch_s * 1e3,
                      "phases": phase_roofline},
         "cpu_baseline": cpu,
         "e2e": e2e,
-        "gpu_launches": args.steps * (launches_per_run(S, prec == sl.SL_FP64 and args.kernel != 1)
-                                      + (S - 1 if split else 0)),
+        "gpu_launches": args.steps * (run_launches(S, prec == sl.SL_FP64, bool(split), steady) if args.kernel != 1
+                                      else launches_per_run(S, False)),
         "clocks": clocks,
         "walk": {"first_run_mean_hops_per_node_update": stats["walk_moves"] / max(1, stats["node_updates"]),
                  "max_hops": stats["max_moves"], "exact_tests": stats["exact_tests"],
