@@ -858,13 +858,17 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
             all_steady = mark_steady(m, n_steps, split_step(m, false), fh);
             if (m->n_problems > 1) {
                 // (a single problem's constants are kernel parameters.)  A
-                // synchronous copy: a graph recorded below may replay them later
+                // synchronous copy: a graph recorded below may replay them
+                // later.  The one before reads the same buffer, rewritten here
+                // and perhaps replaced.
+                g.valid = false;
                 SL_CUDA(cudaStreamSynchronize(s));
                 sl_status st = ensure_fprobs(m, fper * n_steps);
                 if (st != SL_OK) return st;
                 SL_CUDA(cudaMemcpy(m->d.fprobs, fh.data(), fper * n_steps, cudaMemcpyHostToDevice));
             }
         } else {
+            g.valid = false;     // likewise
             SL_CUDA(cudaStreamSynchronize(s));
             sl_status st = ensure_probs(m, per * n_steps);
             if (st != SL_OK) return st;
