@@ -26,6 +26,9 @@
  *     launching are returned at once, conditions found by the kernels (a walk
  *     that gave up) are reported by sl_mesh_status() or sl_run().
  *   - A mesh handle may be used by one stream at a time.
+ *   - A stream that is being captured into a caller's graph is taken by
+ *     sl_step_noalloc alone; a step or run launched on it is refused
+ *     (SL_E_CUDA).
  */
 #ifndef SL_H
 #define SL_H

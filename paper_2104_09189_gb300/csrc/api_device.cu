@@ -702,6 +702,19 @@ static sl_status launch_steady(sl_mesh *m, const FastArgs &a, int config, int32_
     return SL_OK;
 }
 
+// Steps and runs that launch kernels on the caller's stream themselves are not
+// for a stream that is being captured: the caller's graph would keep the
+// address of the step's constants, which later calls rewrite or free, and the
+// node tables, which follow the field.  (sl_run's own graphs end when these
+// change; sl_step_noalloc owns what it hands to its kernels.)
+static sl_status check_not_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    SL_CUDA(cudaStreamIsCapturing(s, &st));
+    if (st != cudaStreamCaptureStatusNone) return fail(SL_E_CUDA, "the stream is being captured (use sl_step_noalloc)");
+    return SL_OK;
+}
+
 static sl_status check_device(const sl_mesh *m)
 {
     int dev = -1;
@@ -851,6 +864,8 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
     std::vector<FastProb> fh;   // the fast kernels' constants, host copy (filled when recording)
     bool all_steady = false;
     if (!reuse) {
+        const sl_status cst = check_not_capturing(s);
+        if (cst != SL_OK) return cst;
         if (fast) {
             fh.resize((size_t)m->n_problems * (size_t)n_steps);
             for (int32_t k = 0; k < n_steps; ++k)
@@ -989,6 +1004,7 @@ extern "C" sl_status sl_step(sl_mesh *m, const sl_problem *probs, int64_t n, con
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<ProbStep> host(m->n_problems);
     st = fill_step(m, probs, n, host.data());
+    if (st == SL_OK) st = check_not_capturing(s);
     if (st != SL_OK) return st;
     const bool debug = dbg && (dbg->feet || dbg->tri || dbg->moves || dbg->flags || dbg->feet_lo);
     if (!use_fast(m)) {

@@ -78,3 +78,26 @@ def test_a_launched_run_between_replays_of_a_batch(eager_steps, kernel):
         sl.sl_mesh_reset_t0(b.h)
         sl.sl_run(b.h, A, 0, 6, v, w, use_graph=True)
         assert bool((v == want[0]).all()) and bool((t0_of(b.h, v.numel()) == want[1]).all()), use
+
+
+@pytest.mark.parametrize("problems", [1, 3])
+@pytest.mark.parametrize("call", ["step", "run"])
+def test_a_capturing_stream_is_refused(call, problems):
+    """A caller's graph would keep addresses of the handle's constants, which
+    later calls rewrite or free, and its tables, which follow the field."""
+    import torch
+    b = Batch((20, 33, 9)[:problems])
+    probs = fields_of(("rotation",) * problems)
+    w = torch.empty_like(b.v0)
+    if call == "run":
+        sl.sl_mesh_set_option(b.h, sl.SL_OPT_ASYNC, 1)
+    sl.sl_step(b.h, probs, 0, b.v0, w)                 # everything a step allocates
+    torch.cuda.synchronize()
+    with torch.cuda.graph(torch.cuda.CUDAGraph(), capture_error_mode="thread_local"):
+        if call == "step":
+            got = status_of(sl.sl_step, b.h, probs, 1, b.v0, w)
+        else:
+            got = status_of(sl.sl_run, b.h, probs, 1, 2, b.v0, w, use_graph=False, stats=False)
+    assert got == sl.SL_E_CUDA
+    sl.sl_step(b.h, probs, 1, b.v0, w)                 # the handle goes on
+    sl.sl_mesh_status(b.h)
