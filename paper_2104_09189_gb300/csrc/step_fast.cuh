@@ -84,7 +84,8 @@ struct FastArgs {
     int32_t nprob;
     int32_t walk_cap;
     int32_t lean_moves;           // FP64: certified moves a lean pass may add to its hops (8; 0 under a
-                                  // hop cap of the caller's, which the hops alone keep to)
+                                  // hop cap of the caller's, which the hops alone keep to: no known
+                                  // triangles then either)
     int64_t N;
     uint32_t *status;
     unsigned long long *stats;

@@ -959,8 +959,9 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     int w0 = tq.y, w1 = tq.z, w2 = tq.w;
     // A foot that ends as its node's coordinate pair, within rounding of the
     // node, is a point of the mesh alone, and its triangle is known (k_pair_tri;
-    // without kLean it is walked to).
-    const int32_t known = kLean && foot_on_pair(a.xyq[i], X, Y) ? a.pair_tri[i] : -1;
+    // without kLean it is walked to, as under a hop cap of the caller's, which
+    // the way there from a far T^0 has to keep to).
+    const int32_t known = kLean && a.lean_moves > 0 && foot_on_pair(a.xyq[i], X, Y) ? a.pair_tri[i] : -1;
     bool ids = true;           // w0..w2 are the vertex ids of the current triangle
     const uint32_t cap = (uint32_t)a.walk_cap;
     uint32_t &hops = c.hops;

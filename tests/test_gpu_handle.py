@@ -101,3 +101,36 @@ def test_a_capturing_stream_is_refused(call, problems):
     assert got == sl.SL_E_CUDA
     sl.sl_step(b.h, probs, 1, b.v0, w)                 # the handle goes on
     sl.sl_mesh_status(b.h)
+
+
+@pytest.mark.parametrize("precision,records,split", [(sl.SL_FP64, 0, 0), (sl.SL_FP64, 1, 0), (sl.SL_FP64, 0, 1),
+                                                     (sl.SL_FP32, 0, 0)],
+                         ids=["fp64", "fp64-records8", "fp64-split", "fp32"])
+def test_every_hop_cap_where_the_field_vanishes(precision, records, split):
+    """The swirl's feet are their nodes at t = 1/2, cells away from the triangles
+    of the step before: the walk back there keeps to a cap of the caller's, the
+    same with and without the counting variant."""
+    m = si.grid_mesh(60, 0.25, 7)
+    g = DeviceRun(m, si.swirl_field(), 0.05, precision=precision)
+    sl.sl_mesh_set_option(g.h, sl.SL_OPT_RECORDS, records)
+    sl.sl_mesh_set_option(g.h, sl.SL_OPT_SPLIT, split)
+    t = g.torch
+    v = g.to_dev(si.cosine_bump(m.xy))
+    w = t.empty_like(v)
+    sl.sl_step(g.h, g.probs, 1, v, w)
+    start = t0_of(g.h, m.n_nodes)
+    outcomes = set()
+    for cap in range(1, 13):
+        sl.sl_mesh_set_option(g.h, sl.SL_OPT_WALK_CAP, cap)
+        got = []
+        for debug in (True, False):
+            sl.sl_mesh_set_t0(g.h, start)
+            w = t.empty_like(v)
+            moves = t.zeros(m.n_nodes, dtype=t.int32, device=g.dev)
+            sl.sl_step(g.h, g.probs, 9, v, w, debug={"moves": moves} if debug else None)
+            got.append((status_of(sl.sl_mesh_status, g.h), w, t0_of(g.h, m.n_nodes)))
+        assert got[0][0] == got[1][0], f"cap {cap}"
+        outcomes.add(got[0][0])
+        if got[0][0] == sl.SL_OK:
+            assert bool((got[0][1] == got[1][1]).all()) and bool((got[0][2] == got[1][2]).all()), f"cap {cap}"
+    assert outcomes == {sl.SL_OK, sl.SL_E_WALK_LIMIT}
