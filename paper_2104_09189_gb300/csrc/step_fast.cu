@@ -111,18 +111,32 @@ void launch_fast_df(const FastArgs &a, bool stats, bool debug, int config, cudaS
 // (foot, certified test, quotient; also 48 bytes, 290 instructions, 64 bytes of
 // gathered vertices) took 0.180 ms.  A 50-step rotation 9.60 -> 6.69 ms.  The
 // weights past L1: they are read once.
+//
+// A node without weights yet (emit_open) takes the full node step, inline: called
+// out of line it put saved registers on every node's path (50 steps 6.64 -> 6.73
+// to 7.46 ms, four forms), inline the spills are its own (6.64 ms).
+template <bool kCompact>
 __global__ void __launch_bounds__(256, 8) k_apply_df(const __grid_constant__ FastArgs a)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_launch_dependents();
     pdl_wait();
-    if (i < a.N) put_value(a, i, apply_weights(a, i));
+    if (i >= a.N) return;
+    float2 v;
+    if (apply_weights(a, i, v)) {
+        put_value(a, i, v);
+        return;
+    }
+    NodeCounters c;
+    step_node<false, true, false, kCompact>(a, i, a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i), c);
 }
 
 void launch_apply_df(const FastArgs &a, cudaStream_t s)
 {
     const unsigned grid = (unsigned)((a.N + 255) / 256);
-    if (grid) launch_step_kernel(k_apply_df, grid, 256, s, a);
+    if (grid == 0) return;
+    if (a.he8) launch_step_kernel(k_apply_df<true>, grid, 256, s, a);
+    else launch_step_kernel(k_apply_df<false>, grid, 256, s, a);
 }
 
 // The triangle that holds node i's coordinate pair, the point a foot of no

@@ -468,6 +468,15 @@ __device__ __forceinline__ void emit_own(const FastArgs &a, int64_t i)
     a.wt[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 }
 
+// A node whose walk gave up has no triangle yet: the next step walks on from
+// where this one stopped (T^0), in the full node step, and stores the weights
+// once it gets there.  Marked by a bound below zero, which every value exceeds,
+// so that the other nodes of those steps pay nothing for it.
+__device__ __forceinline__ void emit_open(const FastArgs &a, int64_t i)
+{
+    a.wq[i] = make_int4((int)i, (int)i, (int)i, __float_as_int(-1.0f));
+}
+
 // V^n is steep in the triangle (SL_OPT_PRECISE): max_k (v_k - v_3)^2 >
 // G^2 den on the high parts, den twice the area, so that max |v_k - v_3| / sqrt(den)
 // -- about the P1 gradient -- exceeds G.  The double-float value is then off
@@ -535,8 +544,9 @@ static __device__ __noinline__ float2 precise_value(const double2 *__restrict__ 
 
 // A later step of a steady field (emit_weights): V = v3 + theta_1 (v1 - v3) +
 // theta_2 (v2 - v3) in double-float, in FP64 from the coordinates where V^n is
-// steep, as p1_value_of and precise_value.
-__device__ __forceinline__ float2 apply_weights(const FastArgs &a, int64_t i)
+// steep, as p1_value_of and precise_value.  false: the node has no weights yet
+// (emit_open).
+__device__ __forceinline__ bool apply_weights(const FastArgs &a, int64_t i, float2 &out)
 {
     int4 w;
     float4 t;
@@ -553,9 +563,11 @@ __device__ __forceinline__ float2 apply_weights(const FastArgs &a, int64_t i)
     two_sum_f(V2.x, -V3.x, d2h, d2l);
     d2l = __fadd_rn(d2l, __fsub_rn(V2.y, V3.y));
     const float s1 = __fsub_rn(V1.x, V3.x), s2 = __fsub_rn(V2.x, V3.x);
-    if (fmaxf(__fmul_rn(s1, s1), __fmul_rn(s2, s2)) > __int_as_float(w.w)) {
+    if (!(fmaxf(__fmul_rn(s1, s1), __fmul_rn(s2, s2)) <= __int_as_float(w.w))) {
+        if (__int_as_float(w.w) < 0.0f) return false;
         const int pi = a.nprob == 1 ? 0 : chunk_problem(a.chunk_prob, a.node_off, i);
-        return precise_value(a.xyd, a.g1, a.g2, a.single ? a.prob0 : a.probs[pi], i, w.x, w.y, w.z, V1, V2, V3);
+        out = precise_value(a.xyd, a.g1, a.g2, a.single ? a.prob0 : a.probs[pi], i, w.x, w.y, w.z, V1, V2, V3);
+        return true;
     }
     const float p1 = __fmul_rn(t.x, d1h), p2 = __fmul_rn(t.z, d2h);
     float q1 = __fmaf_rn(t.x, d1h, -p1), q2 = __fmaf_rn(t.z, d2h, -p2);
@@ -566,7 +578,8 @@ __device__ __forceinline__ float2 apply_weights(const FastArgs &a, int64_t i)
     float ws, wl;
     two_sum_f(p1, p2, ws, wl);
     const df v = df_add(dfp(V3), df_make(ws, __fadd_rn(wl, __fadd_rn(q1, q2))));
-    return make_float2(v.h, v.l);
+    out = make_float2(v.h, v.l);
+    return true;
 }
 
 // A foot that comes out of the foot arithmetic as its own node's stored
@@ -944,7 +957,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     // rounding-sized offset every step.
     if (at_node && (tq.y == (int32_t)i || tq.z == (int32_t)i || tq.w == (int32_t)i)) {
         keep_value(a, i);
-        if (kLean && (P.flags & kFastEmit)) emit_own(a, i);
+        if (kLean && (P.flags & (kFastEmit | kFastUse))) emit_own(a, i);
         if (kExt && a.parent && !a.keep_t0) a.t0v[i] = tq;
         if (kDebug) {
             write_node_foot(a, i);
@@ -1153,8 +1166,9 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
             put_value(a, i, p1_value_of(V1, V2, V3, n1, n2, den));
         }
     }
-    if (kLean && (P.flags & kFastEmit)) {
-        if (at_node && (w0 == (int)i || w1 == (int)i || w2 == (int)i)) emit_own(a, i);
+    if (kLean && (P.flags & (kFastEmit | kFastUse))) {
+        if (!found) emit_open(a, i);
+        else if (at_node && (w0 == (int)i || w1 == (int)i || w2 == (int)i)) emit_own(a, i);
         else emit_weights(a, i, w0, w1, w2, n1, n2, den, flags & SL_NODE_CLIPPED);
     }
     if ((hops > 0 || (kExt && a.parent)) && !(kExt && a.keep_t0))

@@ -112,7 +112,9 @@ __device__ __forceinline__ bool lean_node(const FastArgs &a, int64_t i, int pi)
 {
     const FastProb &P = kSingle ? a.prob0 : a.probs[pi];
     if (!kSingle && (P.flags & kFastUse)) {
-        put_value(a, i, apply_weights(a, i));
+        float2 v;
+        if (!apply_weights(a, i, v)) return false;
+        put_value(a, i, v);
         return true;
     }
     df X, Y;

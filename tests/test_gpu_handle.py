@@ -134,3 +134,28 @@ def test_every_hop_cap_where_the_field_vanishes(precision, records, split):
         if got[0][0] == sl.SL_OK:
             assert bool((got[0][1] == got[1][1]).all()) and bool((got[0][2] == got[1][2]).all()), f"cap {cap}"
     assert outcomes == {sl.SL_OK, sl.SL_E_WALK_LIMIT}
+
+
+@PRECISIONS
+@pytest.mark.parametrize("kinds", [("rotation",), ("rotation", "zero"), ("rotation", "swirl")], ids="+".join)
+@pytest.mark.parametrize("cap,records", [(2, 0), (3, 0), (2, 1)])
+def test_a_steady_run_goes_on_walking_where_a_walk_gave_up(cap, records, kinds, precision):
+    """A node whose walk ends at the caller's cap has no triangle yet: the next
+    steps of a steady run walk on from where it stopped, as the steps of shorter
+    runs do, which locate at every step."""
+    b = Batch((40, 25)[:len(kinds)], precision)
+    sl.sl_mesh_set_option(b.h, sl.SL_OPT_WALK_CAP, cap)
+    sl.sl_mesh_set_option(b.h, sl.SL_OPT_RECORDS, records)
+    probs = fields_of(kinds)
+    a, ta, sa = run_from_start(b.h, probs, b.v0, (3, 3, 2), False)
+    assert sa == sl.SL_E_WALK_LIMIT
+    for _ in range(3):          # launched, recorded, replayed
+        c, tc, sc = run_from_start(b.h, probs, b.v0, (8,), True)
+        assert sc == sa and bool((ta == tc).all())
+        if precision == sl.SL_FP32:
+            assert bool((a == c).all())
+        else:
+            # 2^-43 of |V| and step as in whole runs; where a walk gave up the
+            # value is extrapolated from up to 10 triangle widths away, in two
+            # of the eight steps: errors grow by up to 20^2 < 2^9
+            assert float((a - c).abs().max()) <= 8 * 2.0 ** -34 * float(a.abs().max())
