@@ -422,7 +422,8 @@ sl_status sl_probe_gather(sl_mesh *m, const void *v, void *v_scratch, int32_t re
  * in strategy (b), stores the foot triangle T^f_i there).  t0_dev: device,
  * N int32, global triangle indices in the current numbering, written (get)
  * or read (set) on `stream`; the caller owns it.  With V^n this is the whole
- * state of a run, so a run can stop and resume bitwise.  set validates every
+ * state of a run, so a run can stop and resume bitwise.  SL_E_STATE where the
+ * current device is not the mesh's, as the step calls.  set validates every
  * entry (SL_E_ARG if one is not a triangle of its node's problem; it copies
  * T^0 through the host and synchronises) and refreshes the start-state cache.
  */

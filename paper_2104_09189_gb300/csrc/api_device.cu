@@ -1099,6 +1099,8 @@ extern "C" sl_status sl_run_host(sl_mesh *m, const sl_problem *probs, int64_t n0
 extern "C" sl_status sl_mesh_get_t0(const sl_mesh *m, int32_t *t0_dev, void *stream)
 {
     if (!m || !t0_dev) return fail(SL_E_ARG, "sl_mesh_get_t0: NULL argument");
+    const sl_status st = check_device(m);
+    if (st != SL_OK) return st;
     launch_export_t0((const int4 *)m->d.t0v, t0_dev, m->N, (cudaStream_t)stream);
     SL_CUDA(cudaGetLastError());
     return SL_OK;
@@ -1107,6 +1109,8 @@ extern "C" sl_status sl_mesh_get_t0(const sl_mesh *m, int32_t *t0_dev, void *str
 extern "C" sl_status sl_mesh_set_t0(sl_mesh *m, const int32_t *t0_dev, void *stream)
 {
     if (!m || !t0_dev) return fail(SL_E_ARG, "sl_mesh_set_t0: NULL argument");
+    const sl_status st = check_device(m);
+    if (st != SL_OK) return st;
     std::vector<int32_t> h(m->N);
     SL_CUDA(cudaMemcpyAsync(h.data(), t0_dev, sizeof(int32_t) * m->N, cudaMemcpyDeviceToHost, (cudaStream_t)stream));
     SL_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
@@ -1123,6 +1127,8 @@ extern "C" sl_status sl_mesh_set_t0(sl_mesh *m, const int32_t *t0_dev, void *str
 extern "C" sl_status sl_mesh_reset_t0(sl_mesh *m, void *stream)
 {
     if (!m) return fail(SL_E_ARG, "sl_mesh_reset_t0: mesh is NULL");
+    const sl_status st = check_device(m);
+    if (st != SL_OK) return st;
     m->t0_initial = true;
     launch_reset_t0(m->d.t0_init, (const int4 *)m->d.tri, (int4 *)m->d.t0v, m->N, (cudaStream_t)stream);
     SL_CUDA(cudaGetLastError());

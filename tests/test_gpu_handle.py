@@ -1,5 +1,7 @@
 """GPU tests of what a mesh handle keeps between calls: recorded graphs and
 their constants, steady weights, T^0, options, the tuner, device memory."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -159,3 +161,23 @@ def test_a_steady_run_goes_on_walking_where_a_walk_gave_up(cap, records, kinds, 
             # value is extrapolated from up to 10 triangle widths away, in two
             # of the eight steps: errors grow by up to 20^2 < 2^9
             assert float((a - c).abs().max()) <= 8 * 2.0 ** -34 * float(a.abs().max())
+
+
+def test_t0_calls_want_the_device_of_the_mesh():
+    """As the step calls do.  (One GPU: the handle is told that it belongs to
+    another one; the field's place is checked by what a step answers.)"""
+    import torch
+    b = Batch((12,))
+    probs = fields_of(("rotation",))
+    w = torch.empty_like(b.v0)
+    j = t0_of(b.h, w.numel())
+    # n_problems, N, Nt, precision, device
+    place = ctypes.c_int.from_address(b.h + 28)
+    assert place.value == torch.cuda.current_device()
+    place.value += 1
+    try:
+        got = [status_of(sl.sl_step, b.h, probs, 0, b.v0, w), status_of(sl.sl_mesh_get_t0, b.h, j),
+               status_of(sl.sl_mesh_set_t0, b.h, j), status_of(sl.sl_mesh_reset_t0, b.h)]
+    finally:
+        place.value -= 1
+    assert got == [sl.SL_E_STATE] * 4
