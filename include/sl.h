@@ -139,7 +139,8 @@ typedef enum {
     /* 4 and 6 are not options (SL_E_ARG) */
     SL_OPT_CONFIG = 5,       /* launch configuration of the fast kernels, 0..5: threads per block x
                                 blocks per SM the registers are sized for = 256x4, 128x16, 128x8,
-                                128x9, 256x5, 128x12 (default 5) */
+                                128x9, 256x5, 128x12 (default 5; 1 for FP32 meshes of more nodes
+                                than 12 x 128 per multiprocessor) */
     SL_OPT_CONFIG_FIRST = 7, /* launch configuration for a step whose walks start at the initial
                                 incident triangles (the first step after sl_mesh_create or
                                 sl_mesh_reset_t0): long walks favour fewer resident warps (default 0;

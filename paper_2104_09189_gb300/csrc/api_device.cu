@@ -476,6 +476,7 @@ FastArgs make_fast_args(const sl_mesh *m, const FastProb *fp, const void *vin, v
     a.nprob = m->n_problems;
     a.walk_cap = m->opt_walk_cap > 0 ? m->opt_walk_cap : default_walk_cap(m);
     a.lean_moves = m->opt_walk_cap > 0 ? 0 : 8;
+    a.sms = m->sms;
     a.N = m->N;
     a.status = m->d.status;
     a.stats = m->d.stats;
@@ -860,7 +861,7 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
         g.t0_initial = first_initial;
         g.split = m->opt_split;
     };
-    auto config_of = [&](int32_t k) { return (k == 0 && first_initial) ? first_config(m) : m->opt_config; };
+    auto config_of = [&](int32_t k) { return (k == 0 && first_initial) ? first_config(m) : later_config(m); };
     std::vector<FastProb> fh;   // the fast kernels' constants, host copy (filled when recording)
     bool all_steady = false;
     if (!reuse) {
@@ -1039,14 +1040,14 @@ extern "C" sl_status sl_step(sl_mesh *m, const sl_problem *probs, int64_t n, con
         if (!m->d.dfb) SL_CUDA(cudaMalloc(&m->d.dfb, sizeof(float2) * m->N));
         launch_to_df((const double *)v_in, (float2 *)m->d.dfa, m->N, s);
         FastArgs a = make_fast_args(m, (const FastProb *)m->d.fprobs, m->d.dfa, m->d.dfb, dbg, fh.data());
-        st = launch_fast(m, a, debug, m->opt_config, false, s);
+        st = launch_fast(m, a, debug, later_config(m), false, s);
         if (st != SL_OK) return st;
         launch_from_df((const float2 *)m->d.dfb, (double *)v_out, m->N, s);
         SL_CUDA(cudaGetLastError());
     } else {
         FastArgs a = make_fast_args(m, (const FastProb *)m->d.fprobs, v_in, v_out, dbg, fh.data());
         if (m->precision == SL_FP64) a.io = kIoIn | kIoOut;
-        st = launch_fast(m, a, debug, m->t0_initial ? first_config(m) : m->opt_config, m->t0_initial, s);
+        st = launch_fast(m, a, debug, m->t0_initial ? first_config(m) : later_config(m), m->t0_initial, s);
         if (st != SL_OK) return st;
     }
     m->stepped = true;

@@ -110,7 +110,7 @@ extern "C" sl_status sl_step_noalloc(sl_mesh *m, const sl_problem *probs, int64_
     FastArgs a;
     fast_args_for(m, records, v_in, v_out, nullptr, host, a);
     a.io = kIoIn | kIoOut;
-    launch_fast_df(a, m->opt_stats != 0, false, m->t0_initial ? first_config(m) : m->opt_config, s);
+    launch_fast_df(a, m->opt_stats != 0, false, m->t0_initial ? first_config(m) : later_config(m), s);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(SL_E_CUDA, std::string("sl_step_noalloc: launch: ") + cudaGetErrorString(e));
     m->stepped = true;

@@ -95,7 +95,8 @@ struct sl_mesh {
     int32_t opt_walk_cap = 0;         // 0 = default
     int32_t opt_kernel = 0;
     int32_t opt_block = 0;
-    int32_t opt_config = 5;           // launch configuration of the fast kernels (later steps)
+    int32_t opt_config = -1;          // launch configuration of the fast kernels (later steps; -1: not set,
+                                      // see later_config)
     int32_t opt_config_first = -1;    // ... for a step whose walks start at the initial triangles (-1: not
                                       // set, see first_config)
     int32_t opt_strategy = 0;         // 0 = strategy (b), 1 = strategy (a) (T^0 never overwritten),
@@ -127,6 +128,19 @@ struct sl_mesh {
 };
 
 namespace sl {
+// Nodes above which a step is more than one wave of the chip at 12 blocks of 128
+// per multiprocessor.
+inline bool several_waves(int64_t N, int32_t sms) { return N > (int64_t)sms * 12 * 128; }
+
+// The launch configuration of a later step.  Unset, it is 5 (128 x 12) but for
+// FP32 meshes of more than one wave: 1 (128 x 16) spills there and pays all the
+// same (launch_fast_f32).
+inline int32_t later_config(const sl_mesh *m)
+{
+    if (m->opt_config >= 0) return m->opt_config;
+    return m->precision == SL_FP32 && several_waves(m->N, m->sms) ? 1 : 5;
+}
+
 // The launch configuration of a first step.  Unset, it is 0 (64 registers) for
 // walks of any length, and the later steps' where the jump table shortens them:
 // 8 single steps on 491 k nodes 176 -> 171 us, one on 2 304 nodes 35 -> 31 us a
@@ -134,7 +148,7 @@ namespace sl {
 inline int32_t first_config(const sl_mesh *m)
 {
     if (m->opt_config_first >= 0) return m->opt_config_first;
-    return m->opt_strategy == 0 && m->opt_walk_cap == 0 ? m->opt_config : 0;
+    return m->opt_strategy == 0 && m->opt_walk_cap == 0 ? later_config(m) : 0;
 }
 
 struct FastProb;

@@ -108,6 +108,7 @@ struct FastArgs {
     int32_t *queue;
     uint32_t *queue_count;
     uint32_t *queue_next;         // split steps: the next step's counter, zeroed by the settle pass (or NULL)
+    int32_t sms;                  // host side only: the device's multiprocessors
     // host side only: launch with programmatic stream serialization (the
     // kernel before it on the stream is a step kernel of the same sequence of
     // steps; see launch_step_kernel)

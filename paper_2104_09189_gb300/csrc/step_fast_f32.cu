@@ -18,6 +18,7 @@
 //    exactly;
 //  * theta_1, theta_2 (Eq. 6, relative to vertex 3) and the P1 value are
 //    evaluated in float.
+#include "sl_internal.h"
 #include "predicates.cuh"
 #include "step_common.cuh"
 #include "step_fast.cuh"
@@ -681,18 +682,19 @@ void launch_fast_f32(const FastArgs &a, bool stats, bool debug, int config, cuda
         else launch_f32_cfg<128, 8>(a, stats, debug, s);
         return;
     }
-    // 32 registers (64 warps per SM) spill 16 bytes, which pays where the mesh
-    // fills the chip more than once at 12 blocks per SM: 2048^2 nodes 3.20 -> 2.93
-    // ms per 20 steps, 2.8 M nodes in a batch 4.00 -> 3.58 ms per 50, 478 k nodes
-    // with exclusion 406 -> 333 us per 18; a mesh of one wave (171 k nodes, 30
-    // steps) runs at 858 us with 40 registers and 915 with 32
-    const bool waves = a.N > 152ll * 12 * 128;
+    // 32 registers (64 warps per SM; the lean pass, compiled without the full step,
+    // spills 52 to 68 bytes and reads back 16 to 24, the whole kernel spills 468 to
+    // 512, the rare nodes' full step most of it) pay where the mesh fills the chip
+    // more than once at 12 blocks per SM (several_waves; later_config does the
+    // same for the others): 2048^2 nodes 3.20 -> 2.93 ms per 20 steps, 2.8 M nodes in
+    // a batch 4.00 -> 3.58 ms per 50, 478 k nodes with exclusion 406 -> 333 us per 18;
+    // a mesh of one wave (171 k nodes, 30 steps) runs at 858 us with 40 registers and
+    // 915 with 32
     if (ext) {
-        if (waves) launch_lean_f32_cfg<128, 16, true>(a, s);
+        if (several_waves(a.N, a.sms)) launch_lean_f32_cfg<128, 16, true>(a, s);
         else launch_lean_f32_cfg<128, 8, true>(a, s);
         return;
     }
-    if (config == 5 && waves) config = 1;
     switch (config) {
     case 1: launch_lean_f32_cfg<128, 16>(a, s); break;
     case 2: launch_lean_f32_cfg<128, 8>(a, s); break;

@@ -181,3 +181,37 @@ def test_t0_calls_want_the_device_of_the_mesh():
     finally:
         place.value -= 1
     assert got == [sl.SL_E_STATE] * 4
+
+
+def kernels_of(call):
+    """Names of the kernels a call launches."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    for body in (torch.cuda.synchronize, call):       # a process's first session may record nothing
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            body()
+            torch.cuda.synchronize()
+    return [e.name for e in p.events()]
+
+
+def test_fp32_configurations_of_a_mesh_of_several_waves():
+    """Unset, a mesh of more than one wave takes 128 x 16; every configuration
+    can be had by setting it, 128 x 12 among them."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shapes = {0: "256, 4", 1: "128, 16", 2: "128, 8", 3: "128, 9", 4: "256, 5", 5: "128, 12"}
+    for M, unset in ((40, 5), (int((sms * 12 * 128) ** 0.5) + 5, 1)):
+        m = si.courant_grid(M)
+        g = DeviceRun(m, si.rotation_field(), 0.01, precision=sl.SL_FP32)
+        v = g.to_dev(si.gaussian(m.xy))
+        w = g.torch.empty_like(v)
+        for c in (None, 5, 1, 0, 4):
+            if c is None:
+                assert sl.sl_mesh_get_option(g.h, sl.SL_OPT_CONFIG) == unset
+            else:
+                sl.sl_mesh_set_option(g.h, sl.SL_OPT_CONFIG, c)
+                assert sl.sl_mesh_get_option(g.h, sl.SL_OPT_CONFIG) == c
+            want = f"k_lean_f32<{shapes[unset if c is None else c]},"
+            names = kernels_of(lambda: sl.sl_step(g.h, g.probs, 0, v, w))
+            assert any(want in n for n in names), (M, c, names)
