@@ -145,7 +145,9 @@ typedef enum {
                                 incident triangles (the first step after sl_mesh_create or
                                 sl_mesh_reset_t0): long walks favour fewer resident warps (default 0;
                                 until it is set, a first step that may start at the table of start
-                                triangles, see SL_OPT_WALK_CAP, takes SL_OPT_CONFIG's) */
+                                triangles, see SL_OPT_WALK_CAP, takes SL_OPT_CONFIG's).  Read while
+                                unset, both give the configuration a step would take now, so that
+                                setting what was read changes no launch. */
     SL_OPT_STRATEGY = 8,     /* start triangle of the walks (Sec. 3): 0 = strategy (b), the triangle
                                 found at the previous step (default); 1 = strategy (a), the node's own
                                 incident triangle at every step (T^0 is never overwritten); 2 = the

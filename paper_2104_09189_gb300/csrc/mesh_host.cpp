@@ -456,7 +456,7 @@ extern "C" sl_status sl_mesh_get_option(const sl_mesh *m, int32_t option, int64_
     case SL_OPT_KERNEL: *value = m->opt_kernel; break;
     case SL_OPT_BLOCK: *value = m->opt_block; break;
     case SL_OPT_CONFIG: *value = sl::later_config(m); break;
-    case SL_OPT_CONFIG_FIRST: *value = m->opt_config_first >= 0 ? m->opt_config_first : 0; break;
+    case SL_OPT_CONFIG_FIRST: *value = sl::first_config(m); break;
     case SL_OPT_STRATEGY: *value = m->opt_strategy; break;
     case SL_OPT_OUTSIDE: *value = m->opt_outside; break;
     case SL_OPT_SPLIT: *value = m->opt_split; break;

@@ -215,3 +215,25 @@ def test_fp32_configurations_of_a_mesh_of_several_waves():
             want = f"k_lean_f32<{shapes[unset if c is None else c]},"
             names = kernels_of(lambda: sl.sl_step(g.h, g.probs, 0, v, w))
             assert any(want in n for n in names), (M, c, names)
+
+
+@pytest.mark.parametrize("strategy,cap", [(0, 0), (1, 0), (0, 50)])
+def test_reading_and_setting_the_configurations_changes_no_launch(strategy, cap):
+    """A program that saves its options and sets them again keeps its launches,
+    also while they are unset."""
+    m = si.grid_mesh(40, 0.25, 3)
+    g = DeviceRun(m, si.rotation_field(), 0.01)
+    sl.sl_mesh_set_option(g.h, sl.SL_OPT_STRATEGY, strategy)
+    sl.sl_mesh_set_option(g.h, sl.SL_OPT_WALK_CAP, cap)
+    v = g.to_dev(si.gaussian(m.xy))
+    w = g.torch.empty_like(v)
+
+    def steps():
+        sl.sl_mesh_reset_t0(g.h)
+        sl.sl_step(g.h, g.probs, 0, v, w)
+        sl.sl_step(g.h, g.probs, 1, v, w)
+
+    before = [n for n in kernels_of(steps) if "k_lean" in n]
+    for option in (sl.SL_OPT_CONFIG, sl.SL_OPT_CONFIG_FIRST):
+        sl.sl_mesh_set_option(g.h, option, sl.sl_mesh_get_option(g.h, option))
+    assert len(before) == 2 and [n for n in kernels_of(steps) if "k_lean" in n] == before
