@@ -377,7 +377,9 @@ typedef struct {
  * step and 49 later ones) is faster.  v (device, N values,
  * V^0) and v_scratch (device, N values) are used as in sl_run; v, T^0 and
  * the statistics counters are restored before returning (the call
- * synchronises and allocates temporary device buffers).  No counterpart in
+ * synchronises and allocates temporary device buffers).  Every timed step
+ * locates its feet, also where a run of steady fields would find them once
+ * for all its steps: those steps have one launch shape.  No counterpart in
  * the paper: it tunes the launch shape of the fused step.
  */
 sl_status sl_autotune(sl_mesh *m, const sl_problem *probs, int32_t probe_steps, void *v, void *v_scratch,

@@ -803,8 +803,10 @@ static bool mark_steady(sl_mesh *m, int32_t n_steps, bool split_rest, std::vecto
     return all;
 }
 
+// weights: steady fields may keep them (mark_steady); the tuners time steps that
+// locate, which differ in what they choose between
 static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int32_t n_steps, void *v, void *v2,
-                           int32_t use_graph, cudaStream_t s)
+                           int32_t use_graph, cudaStream_t s, bool weights = true)
 {
     const bool fast = use_fast(m);
     // strategy (c) launches once per spanning-tree level and step: far too
@@ -871,7 +873,7 @@ static sl_status run_steps(sl_mesh *m, const sl_problem *probs, int64_t n0, int3
             fh.resize((size_t)m->n_problems * (size_t)n_steps);
             for (int32_t k = 0; k < n_steps; ++k)
                 fill_fast(m, host.data() + (size_t)k * m->n_problems, fh.data() + (size_t)k * m->n_problems);
-            all_steady = mark_steady(m, n_steps, split_step(m, false), fh);
+            all_steady = weights && mark_steady(m, n_steps, split_step(m, false), fh);
             if (m->n_problems > 1) {
                 // (a single problem's constants are kernel parameters.)  A
                 // synchronous copy: a graph recorded below may replay them
@@ -1289,10 +1291,10 @@ extern "C" sl_status sl_autotune_layout(sl_mesh *m, const sl_problem *probs, int
         if (r == SL_OK) r = sl_mesh_reset_t0(m, s);
         if (r != SL_OK) return r;
         SL_CUDA(cudaEventRecord(e0, s));
-        r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s);
+        r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s, false);
         if (r != SL_OK) return r;
         m->t0_initial = false;
-        r = run_steps(m, probs, 1, probe_steps, v, v_scratch, 0, s);
+        r = run_steps(m, probs, 1, probe_steps, v, v_scratch, 0, s, false);
         if (r != SL_OK) return r;
         SL_CUDA(cudaEventRecord(e1, s));
         SL_CUDA(cudaEventSynchronize(e1));
@@ -1424,7 +1426,7 @@ extern "C" sl_status sl_autotune(sl_mesh *m, const sl_problem *probs, int32_t pr
         m->opt_split = 0;
         {   // one untimed step first: lazy module loading and first-touch costs
             sl_status r = sl_mesh_reset_t0(m, s);
-            if (r == SL_OK) r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s);
+            if (r == SL_OK) r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s, false);
             if (r != SL_OK) return r;
             SL_CUDA(cudaStreamSynchronize(s));
         }
@@ -1434,11 +1436,11 @@ extern "C" sl_status sl_autotune(sl_mesh *m, const sl_problem *probs, int32_t pr
             sl_status r = sl_mesh_reset_t0(m, s);
             if (r != SL_OK) return r;
             SL_CUDA(cudaEventRecord(e0, s));
-            r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s);
+            r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s, false);
             if (r != SL_OK) return r;
             m->t0_initial = false;
             SL_CUDA(cudaEventRecord(e1, s));
-            r = run_steps(m, probs, 1, probe_steps, v, v_scratch, 0, s);
+            r = run_steps(m, probs, 1, probe_steps, v, v_scratch, 0, s, false);
             if (r != SL_OK) return r;
             SL_CUDA(cudaEventRecord(e2, s));
             SL_CUDA(cudaEventSynchronize(e2));
@@ -1463,11 +1465,11 @@ extern "C" sl_status sl_autotune(sl_mesh *m, const sl_problem *probs, int32_t pr
                 SL_CUDA(cudaMemcpyAsync(v, v_save, vbytes, cudaMemcpyDeviceToDevice, s));
                 r = sl_mesh_reset_t0(m, s);
                 if (r != SL_OK) return r;
-                r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s);
+                r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s, false);
                 if (r != SL_OK) return r;
                 m->t0_initial = false;
                 SL_CUDA(cudaEventRecord(e1, s));
-                r = run_steps(m, probs, 1, probe_steps, v, v_scratch, 0, s);
+                r = run_steps(m, probs, 1, probe_steps, v, v_scratch, 0, s, false);
                 if (r != SL_OK) return r;
                 SL_CUDA(cudaEventRecord(e2, s));
                 SL_CUDA(cudaEventSynchronize(e2));
@@ -1500,11 +1502,11 @@ extern "C" sl_status sl_autotune(sl_mesh *m, const sl_problem *probs, int32_t pr
                 r = sl_mesh_reset_t0(m, s);
                 if (r != SL_OK) return r;
                 SL_CUDA(cudaEventRecord(e0, s));
-                r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s);
+                r = run_steps(m, probs, 0, 1, v, v_scratch, 0, s, false);
                 if (r != SL_OK) return r;
                 m->t0_initial = false;
                 SL_CUDA(cudaEventRecord(e1, s));
-                r = run_steps(m, probs, 1, probe_steps, v, v_scratch, 0, s);
+                r = run_steps(m, probs, 1, probe_steps, v, v_scratch, 0, s, false);
                 if (r != SL_OK) return r;
                 SL_CUDA(cudaEventRecord(e2, s));
                 SL_CUDA(cudaEventSynchronize(e2));

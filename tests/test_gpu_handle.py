@@ -237,3 +237,15 @@ def test_reading_and_setting_the_configurations_changes_no_launch(strategy, cap)
     for option in (sl.SL_OPT_CONFIG, sl.SL_OPT_CONFIG_FIRST):
         sl.sl_mesh_set_option(g.h, option, sl.sl_mesh_get_option(g.h, option))
     assert len(before) == 2 and [n for n in kernels_of(steps) if "k_lean" in n] == before
+
+
+@PRECISIONS
+def test_the_tuner_times_steps_that_locate(precision):
+    """With a steady field and any number of probe steps: what it chooses is for
+    steps that locate; the others run in one form whatever it chooses."""
+    m = si.grid_mesh(120, 0.25, 3)
+    g = DeviceRun(m, si.rotation_field(), 0.01, precision=precision)
+    v = g.to_dev(si.gaussian(m.xy))
+    w = g.torch.empty_like(v)
+    names = kernels_of(lambda: sl.sl_autotune(g.h, g.probs, 8, v, w))
+    assert any("k_lean" in n for n in names) and not any("k_apply" in n for n in names)
