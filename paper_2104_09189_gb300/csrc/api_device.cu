@@ -113,8 +113,8 @@ void free_device(sl_mesh *m)
 {
     release_l2_window(m);
     DeviceMesh &d = m->d;
-    void *ptrs[] = {d.xy, d.tv[0], d.tv[1], d.tv[2], d.tn[0], d.tn[1], d.tn[2], d.t0, d.t0_init, d.pair_tri, d.t0v, d.node_off, d.chunk_prob,
-                    d.status, d.probs, d.fprobs, d.xyq, d.xyh, d.g1, d.g2, d.tparams, d.dfa, d.dfb, d.he, d.he8, d.wq, d.wt, d.tri, d.jump, d.grid_t0v, d.tree_order, d.tree_parent, d.queue, d.queue_count,
+    void *ptrs[] = {d.xy, d.tv[0], d.tv[1], d.tv[2], d.tn[0], d.tn[1], d.tn[2], d.t0, d.t0_init, d.extras, d.t0v, d.node_off, d.chunk_prob,
+                    d.status, d.probs, d.fprobs, d.xyq, d.xyh, d.g1, d.g2, d.tparams, d.dfa, d.dfb, d.he, d.he8, d.weights, d.grid_t0v, d.tree_order, d.tree_parent, d.queue, d.queue_count,
                     m->host_v, m->host_v2};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -148,6 +148,7 @@ static float hop_edge_bound(const sl_mesh *m, const std::vector<float2> &h)
     return (double)f >= L ? f : std::nextafter(f, __builtin_inff());
 }
 
+static sl_status alloc_extras(sl_mesh *m);
 static sl_status build_jump_table(sl_mesh *m);
 
 // Copy the host arrays (current numbering) to the device, converting local
@@ -206,8 +207,6 @@ static sl_status upload_arrays(sl_mesh *m)
     // half-edge walk records of the fast kernels
     sl_status st = build_walk_records(m);
     if (st != SL_OK) return st;
-    launch_build_tri(d.tv, Nt, (int4 *)d.tri, 0);
-    SL_CUDA(cudaGetLastError());
     SL_CUDA(cudaMemcpy(d.t0, m->t0.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice));
     SL_CUDA(cudaMemcpy(d.t0_init, m->t0_init.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice));
     SL_CUDA(cudaMemcpy(d.node_off, m->node_off.data(), sizeof(int64_t) * (m->n_problems + 1), cudaMemcpyHostToDevice));
@@ -226,10 +225,13 @@ static sl_status upload_arrays(sl_mesh *m)
         if (!d.chunk_prob) SL_CUDA(cudaMalloc(&d.chunk_prob, sizeof(int2) * nc));
         SL_CUDA(cudaMemcpy(d.chunk_prob, cp.data(), sizeof(int2) * nc, cudaMemcpyHostToDevice));
     }
+    st = alloc_extras(m);
+    if (st != SL_OK) return st;
+    launch_build_tri(d.tv, Nt, (int4 *)d.tri, 0);
+    SL_CUDA(cudaGetLastError());
     st = build_jump_table(m);
     if (st != SL_OK) return st;
     if (m->precision == SL_FP64) {
-        if (!d.pair_tri) SL_CUDA(cudaMalloc(&d.pair_tri, sizeof(int32_t) * N));
         launch_pair_tri(make_fast_args(m, nullptr, nullptr, nullptr, nullptr), d.pair_tri, 0);
         SL_CUDA(cudaGetLastError());
     }
@@ -239,28 +241,71 @@ static sl_status upload_arrays(sl_mesh *m)
     return SL_OK;
 }
 
-// The jump table of every problem: a grid of about one cell per four nodes,
-// built on the device (its scratch is the start-state cache, 16 bytes per
-// node, filled afterwards: 2 bytes per node of seeds and two integers per
-// problem of at least 3 nodes).
-static sl_status build_jump_table(sl_mesh *m)
+static size_t line_up(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
+
+// Bytes of the weights of a run's steady fields (emit_weights).
+static size_t weight_bytes(const sl_mesh *m)
+{
+    return line_up(sizeof(int4) * (size_t)m->N) +
+           line_up((m->precision == SL_FP64 ? sizeof(float4) : sizeof(float)) * (size_t)m->N);
+}
+
+static void place_weights(sl_mesh *m, void *base)
+{
+    m->d.wq = base;
+    m->d.wt = (char *)base + line_up(sizeof(int4) * (size_t)m->N);
+}
+
+// Up to this many nodes a handle has room for its weights from the start: an
+// allocation takes 50 to 100 us whatever its size, which a first run of a few
+// steps does not earn back (the first 10 steps of a rotation without weights,
+// with weights allocated in the run, and with room from the start: 50 k nodes
+// 110, 191 and 89 us, 200 k 126, 263 and 102, 1 M 272, 351 and 201; 2.3 M nodes in
+// FP32, 4 steps, still 442 allocating them where locating at every step took
+// 361).  Larger meshes allocate it in the first run that uses it (ensure_weights).
+constexpr int64_t kEagerWeights = 1 << 22;
+
+// The problems' grids of the jump table, about one cell per four nodes, and the
+// arrays that follow from the mesh, in one allocation.
+static sl_status alloc_extras(sl_mesh *m)
 {
     DeviceMesh &d = m->d;
     const int32_t np = m->n_problems;
+    if (d.extras) return SL_OK;     // a renumbering: the same sizes
     m->jump_g.resize(np);
     m->jump_off.resize(np + 1);
     int64_t cells = 0;
-    int32_t max_g = 1;
     for (int32_t p = 0; p < np; ++p) {
         const double n = (double)(m->node_off[p + 1] - m->node_off[p]);
         const int32_t g = std::max(1, (int32_t)(0.5 * std::sqrt(n)));
         m->jump_g[p] = g;
         m->jump_off[p] = (int32_t)cells;
         cells += (int64_t)g * g;
-        max_g = std::max(max_g, g);
     }
     m->jump_off[np] = (int32_t)cells;     // at most a quarter of the nodes: an int32
-    if (!d.jump) SL_CUDA(cudaMalloc(&d.jump, sizeof(int4) * (size_t)cells));
+    // (on 256 bytes each: a warp's 512 bytes of weights from the middle of a line
+    // are a line more, 1.5 % of a run)
+    const size_t tri = line_up(sizeof(int4) * (size_t)m->Nt), jump = line_up(sizeof(int4) * (size_t)cells),
+                 pair = m->precision == SL_FP64 ? sizeof(int32_t) * (size_t)m->N : 0,
+                 w = m->N <= kEagerWeights ? weight_bytes(m) : 0;
+    SL_CUDA(cudaMalloc(&d.extras, tri + jump + w + pair));
+    char *p = (char *)d.extras;
+    d.tri = p;
+    d.jump = p += tri;
+    p += jump;
+    if (w) place_weights(m, p);
+    if (pair) d.pair_tri = (int32_t *)(p + w);
+    return SL_OK;
+}
+
+// The jump table of every problem, built on the device (its scratch is the
+// start-state cache, 16 bytes per node, filled afterwards: 2 bytes per node of
+// seeds and two integers per problem of at least 3 nodes).
+static sl_status build_jump_table(sl_mesh *m)
+{
+    DeviceMesh &d = m->d;
+    const int32_t np = m->n_problems;
+    const int64_t cells = m->jump_off[np];
     uint32_t *seed = (uint32_t *)d.t0v;
     int32_t *off = (int32_t *)(seed + 2 * (size_t)cells);
     std::vector<int32_t> hg(m->jump_off);
@@ -278,7 +323,7 @@ static sl_status build_jump_table(sl_mesh *m)
     a.gp = off + np + 1;
     a.nprob = np;
     a.cells = (int32_t)cells;
-    a.max_g = max_g;
+    a.max_g = *std::max_element(m->jump_g.begin(), m->jump_g.end());
     a.N = m->N;
     a.seed[0] = seed;
     a.seed[1] = a.seed[0] + cells;
@@ -335,7 +380,6 @@ sl_status upload(sl_mesh *m)
         SL_CUDA(cudaMalloc(&d.tv[k], sizeof(int32_t) * Nt));
         SL_CUDA(cudaMalloc(&d.tn[k], sizeof(int32_t) * Nt));
     }
-    SL_CUDA(cudaMalloc(&d.tri, sizeof(int4) * (Nt > 0 ? Nt : 1)));
     SL_CUDA(cudaMalloc(&d.t0, sizeof(int32_t) * N));
     if (m->precision == SL_FP64) SL_CUDA(cudaMalloc(&d.xyh, sizeof(float2) * N));
     SL_CUDA(cudaMalloc(&d.t0_init, sizeof(int32_t) * N));
@@ -769,6 +813,20 @@ static sl_status ensure_fprobs(sl_mesh *m, size_t bytes)
     return SL_OK;
 }
 
+// Room for the weights (kEagerWeights); false: there is none, and the steps
+// locate every time.
+static bool ensure_weights(sl_mesh *m)
+{
+    if (m->d.wq) return true;
+    if (cudaMalloc(&m->d.weights, weight_bytes(m)) != cudaSuccess) {
+        cudaGetLastError();
+        m->d.weights = nullptr;
+        return false;
+    }
+    place_weights(m, m->d.weights);
+    return true;
+}
+
 // Steady fields of a run (emit_weights): problems whose constants are the same
 // at every one of the n_steps steps store their weights at the first step and
 // use them at the others.  Marks them in fh and returns whether all of them
@@ -790,14 +848,7 @@ static bool mark_steady(sl_mesh *m, int32_t n_steps, bool split_rest, std::vecto
         all &= steady[p] != 0;
     }
     if (!any || (split_rest && !all)) return false;
-    if (!m->d.wq || !m->d.wt) {
-        const size_t tsz = m->precision == SL_FP64 ? sizeof(float4) : sizeof(float);
-        if ((!m->d.wq && cudaMalloc(&m->d.wq, sizeof(int4) * m->N) != cudaSuccess) ||
-            (!m->d.wt && cudaMalloc(&m->d.wt, tsz * m->N) != cudaSuccess)) {
-            cudaGetLastError();     // no room: the steps locate every time
-            return false;
-        }
-    }
+    if (!ensure_weights(m)) return false;
     for (int32_t p = 0; p < np; ++p)
         for (int32_t k = 0; k < n_steps && steady[p]; ++k) fh[(size_t)k * np + p].flags |= k == 0 ? kFastEmit : kFastUse;
     return all;

@@ -33,6 +33,8 @@ struct DeviceMesh {
                                                     // boundary: -1 - side (0: x=0, 1: x=1, 2: y=0, 3: y=1)
     int32_t *t0 = nullptr;            // staging of T^0 as triangle indices (global) to and from the host
     int32_t *t0_init = nullptr;       // the initial start triangles (global)
+    void *extras = nullptr;           // one allocation: tri, jump, pair_tri and, up to kEagerWeights nodes, the
+                                      // weights
     int32_t *pair_tri = nullptr;      // FP64: the triangle of each node's coordinate pair, or -1
     void *t0v = nullptr;              // T^0: int4 (3 T^0, its vertex ids) per node
     void *grid_t0v = nullptr;         // int4 start state per structured-grid triangle (strategy 2)
@@ -55,6 +57,7 @@ struct DeviceMesh {
     double *tparams = nullptr;        // field parameters the tables were built from (device)
     void *dfa = nullptr, *dfb = nullptr;   // value scratch of sl_step for the fast FP64 kernel
     void *he = nullptr;               // float4 half-edge walk records of the fast kernels (3 Nt), or NULL
+    void *weights = nullptr;          // the weights' allocation where extras does not hold them
     void *wq = nullptr, *wt = nullptr;   // a run's steady weights per node (FastArgs; FP32: wt holds wt2)
     void *tri = nullptr;              // int4 (3 t, its vertex ids) per triangle
     void *jump = nullptr;             // int4 start state per cell of the problems' jump tables

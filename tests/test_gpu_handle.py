@@ -249,3 +249,19 @@ def test_the_tuner_times_steps_that_locate(precision):
     w = g.torch.empty_like(v)
     names = kernels_of(lambda: sl.sl_autotune(g.h, g.probs, 8, v, w))
     assert any("k_lean" in n for n in names) and not any("k_apply" in n for n in names)
+
+
+@PRECISIONS
+@pytest.mark.parametrize("steps", [4, 30])
+def test_the_first_steady_run_of_a_handle_allocates_nothing(steps, precision):
+    """Its weights have their room from the start: an allocation costs such a run
+    more than the weights save."""
+    m = si.grid_mesh(700, 0.25, 3)         # weights of 15 or 9 MiB: seen in what is free
+    g = DeviceRun(m, si.rotation_field(), 0.001, precision=precision)
+    v = g.to_dev(si.gaussian(m.xy))
+    w = g.torch.empty_like(v)
+    sl.sl_run(g.h, g.probs, 0, 1, v, w)
+    before = g.torch.cuda.mem_get_info()[0]
+    names = kernels_of(lambda: sl.sl_run(g.h, g.probs, 1, steps, v, w))
+    assert any("k_apply" in n for n in names)
+    assert g.torch.cuda.mem_get_info()[0] >= before - (4 << 20)
