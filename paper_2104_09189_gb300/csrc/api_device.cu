@@ -148,7 +148,7 @@ static float hop_edge_bound(const sl_mesh *m, const std::vector<float2> &h)
     return (double)f >= L ? f : std::nextafter(f, __builtin_inff());
 }
 
-static sl_status alloc_extras(sl_mesh *m);
+static void alloc_extras(sl_mesh *m);
 static sl_status build_jump_table(sl_mesh *m);
 
 // Copy the host arrays (current numbering) to the device, converting local
@@ -225,13 +225,14 @@ static sl_status upload_arrays(sl_mesh *m)
         if (!d.chunk_prob) SL_CUDA(cudaMalloc(&d.chunk_prob, sizeof(int2) * nc));
         SL_CUDA(cudaMemcpy(d.chunk_prob, cp.data(), sizeof(int2) * nc, cudaMemcpyHostToDevice));
     }
-    st = alloc_extras(m);
-    if (st != SL_OK) return st;
-    launch_build_tri(d.tv, Nt, (int4 *)d.tri, 0);
-    SL_CUDA(cudaGetLastError());
-    st = build_jump_table(m);
-    if (st != SL_OK) return st;
-    if (m->precision == SL_FP64) {
+    alloc_extras(m);
+    if (d.extras) {
+        launch_build_tri(d.tv, Nt, (int4 *)d.tri, 0);
+        SL_CUDA(cudaGetLastError());
+        st = build_jump_table(m);
+        if (st != SL_OK) return st;
+    }
+    if (d.pair_tri) {
         launch_pair_tri(make_fast_args(m, nullptr, nullptr, nullptr, nullptr), d.pair_tri, 0);
         SL_CUDA(cudaGetLastError());
     }
@@ -265,13 +266,33 @@ static void place_weights(sl_mesh *m, void *base)
 // 361).  Larger meshes allocate it in the first run that uses it (ensure_weights).
 constexpr int64_t kEagerWeights = 1 << 22;
 
+// Arrays that only make the steps faster: allocated where kSpareBytes per node
+// stay free beside them, what a caller's buffers and the handle's later ones
+// (tables 32, values 32, queue 4) may still need.  NULL otherwise, and the handle
+// does without.
+#ifndef SL_SPARE_BYTES      // a build that never has room for them sets more than any device has
+#define SL_SPARE_BYTES 128
+#endif
+constexpr size_t kSpareBytes = SL_SPARE_BYTES;
+static void *optional_malloc(const sl_mesh *m, size_t bytes)
+{
+    size_t avail = 0, total = 0;
+    void *p = nullptr;
+    if (cudaMemGetInfo(&avail, &total) == cudaSuccess && avail >= bytes + kSpareBytes * (size_t)m->N &&
+        cudaMalloc(&p, bytes) == cudaSuccess)
+        return p;
+    cudaGetLastError();
+    return nullptr;
+}
+
 // The problems' grids of the jump table, about one cell per four nodes, and the
-// arrays that follow from the mesh, in one allocation.
-static sl_status alloc_extras(sl_mesh *m)
+// arrays that follow from the mesh, in one allocation.  Without them (d.tri is
+// NULL) every step is the full node step.
+static void alloc_extras(sl_mesh *m)
 {
     DeviceMesh &d = m->d;
     const int32_t np = m->n_problems;
-    if (d.extras) return SL_OK;     // a renumbering: the same sizes
+    if (d.extras) return;           // a renumbering: the same sizes
     m->jump_g.resize(np);
     m->jump_off.resize(np + 1);
     int64_t cells = 0;
@@ -288,14 +309,15 @@ static sl_status alloc_extras(sl_mesh *m)
     const size_t tri = line_up(sizeof(int4) * (size_t)m->Nt), jump = line_up(sizeof(int4) * (size_t)cells),
                  pair = m->precision == SL_FP64 ? sizeof(int32_t) * (size_t)m->N : 0,
                  w = m->N <= kEagerWeights ? weight_bytes(m) : 0;
-    SL_CUDA(cudaMalloc(&d.extras, tri + jump + w + pair));
+    d.extras = w ? optional_malloc(m, tri + jump + pair + w) : nullptr;
+    const bool weights = d.extras != nullptr;
+    if (!d.extras) d.extras = optional_malloc(m, tri + jump + pair);
+    if (!d.extras) return;
     char *p = (char *)d.extras;
     d.tri = p;
-    d.jump = p += tri;
-    p += jump;
-    if (w) place_weights(m, p);
-    if (pair) d.pair_tri = (int32_t *)(p + w);
-    return SL_OK;
+    d.jump = p + tri;
+    if (pair) d.pair_tri = (int32_t *)(p + tri + jump + (weights ? w : 0));
+    if (weights) place_weights(m, p + tri + jump);
 }
 
 // The jump table of every problem, built on the device (its scratch is the
@@ -818,11 +840,8 @@ static sl_status ensure_fprobs(sl_mesh *m, size_t bytes)
 static bool ensure_weights(sl_mesh *m)
 {
     if (m->d.wq) return true;
-    if (cudaMalloc(&m->d.weights, weight_bytes(m)) != cudaSuccess) {
-        cudaGetLastError();
-        m->d.weights = nullptr;
-        return false;
-    }
+    if (m->d.tri) m->d.weights = optional_malloc(m, weight_bytes(m));
+    if (!m->d.weights) return false;
     place_weights(m, m->d.weights);
     return true;
 }
@@ -1184,7 +1203,10 @@ extern "C" sl_status sl_mesh_reset_t0(sl_mesh *m, void *stream)
     const sl_status st = check_device(m);
     if (st != SL_OK) return st;
     m->t0_initial = true;
-    launch_reset_t0(m->d.t0_init, (const int4 *)m->d.tri, (int4 *)m->d.t0v, m->N, (cudaStream_t)stream);
+    if (m->d.tri)
+        launch_reset_t0(m->d.t0_init, (const int4 *)m->d.tri, (int4 *)m->d.t0v, m->N, (cudaStream_t)stream);
+    else
+        launch_fill_t0v(m->d.t0_init, m->d.tv[0], m->d.tv[1], m->d.tv[2], (int4 *)m->d.t0v, m->N, (cudaStream_t)stream);
     SL_CUDA(cudaGetLastError());
     return SL_OK;
 }

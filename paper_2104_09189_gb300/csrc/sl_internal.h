@@ -34,7 +34,7 @@ struct DeviceMesh {
     int32_t *t0 = nullptr;            // staging of T^0 as triangle indices (global) to and from the host
     int32_t *t0_init = nullptr;       // the initial start triangles (global)
     void *extras = nullptr;           // one allocation: tri, jump, pair_tri and, up to kEagerWeights nodes, the
-                                      // weights
+                                      // weights; NULL where the device has no room for it
     int32_t *pair_tri = nullptr;      // FP64: the triangle of each node's coordinate pair, or -1
     void *t0v = nullptr;              // T^0: int4 (3 T^0, its vertex ids) per node
     void *grid_t0v = nullptr;         // int4 start state per structured-grid triangle (strategy 2)

@@ -79,14 +79,15 @@ void launch_finish_df(const FastArgs &a, bool stats, bool debug, int sms, cudaSt
 // 128 x 8, 3 = 128 x 9 (56 registers), 4 = 256 x 5, 5 = 128 x 12.  Each
 // is instantiated in a translation unit of its own pair (step_fast_c*.cu).
 //
-// They are configurations of the lean kernel.  Statistics, debug outputs and
-// strategy (c) run the full node step in one configuration of its own.  A hop
+// They are configurations of the lean kernel.  Statistics, debug outputs,
+// strategy (c) and a handle without its tables (a.tri) run the full node step in
+// one configuration of its own.  A hop
 // cap of the caller's holds in the lean kernel too: its hops are the full step's
 // and end at the cap (a 1024^2-node swirl of 20 steps under a cap it never meets:
 // 1.33 ms in the full step, 1.22 here).
 void launch_fast_df(const FastArgs &a, bool stats, bool debug, int config, cudaStream_t s)
 {
-    if (stats || debug || a.order) {
+    if (stats || debug || a.order || !a.tri) {
         launch_full_df(a, stats, debug, s);
         return;
     }

@@ -53,7 +53,8 @@ struct FastArgs {
     const float2 *xyh;            // FP64 meshes: high parts (xh, yh) for the FP32 hop tests
     const int32_t *tv[3];
     const int32_t *tn[3];         // -1 - side on the boundary (0: x=0, 1: x=1, 2: y=0, 3: y=1)
-    const int4 *tri;              // per triangle: (3 t, its three vertex ids), the start state of t
+    const int4 *tri;              // per triangle: (3 t, its three vertex ids), the start state of t; NULL
+                                  // (then jump and pair_tri are too): no lean steps
     const float4 *he;             // half-edge walk records, 3 per triangle (k_build_he), or NULL
     const uint2 *he8;             // FP64 meshes whose records fit in 8 bytes (k_build_he8), or NULL
     // Start states (as t0v) of a triangle in or near each cell of a uniform

@@ -9,7 +9,8 @@ void launch_lean_df_ext(const FastArgs &a, cudaStream_t s) { launch_lean_df_cfg<
 
 void launch_full_df(const FastArgs &a, bool stats, bool debug, cudaStream_t s)
 {
-    if (a.exclude || a.order || a.grid_M > 0 || a.keep_t0) launch_fast_df_cfg<128, 8, true>(a, stats, debug, s);
+    // (the plain form of the kernel counts or reports)
+    if (a.exclude || a.order || a.grid_M > 0 || a.keep_t0 || !(stats || debug)) launch_fast_df_cfg<128, 8, true>(a, stats, debug, s);
     else launch_fast_df_cfg<128, 8>(a, stats, debug, s);
 }
 

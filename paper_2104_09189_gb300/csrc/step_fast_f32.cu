@@ -663,22 +663,22 @@ static void launch_f32_cfg(const FastArgs &a, bool stats, bool debug, cudaStream
         else launch_step_kernel(k_step_fast_f32<true, false, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
     } else {
         if (debug) launch_step_kernel(k_step_fast_f32<false, true, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
-        else if constexpr (kExt)    // strategy (c); the lean kernel takes the others
+        else if constexpr (kExt)    // strategy (c), no room for the lean kernel's tables
             launch_step_kernel(k_step_fast_f32<false, false, kBlock, kMinBlocks, kExt>, grid, kBlock, s, a);
     }
 }
 
 void launch_fast_f32(const FastArgs &a, bool stats, bool debug, int config, cudaStream_t s)
 {
-    // statistics, debug outputs and strategy (c): the full node step, one
-    // configuration (128 x 8).  A hop cap of the caller's needs no route of its
+    // statistics, debug outputs, strategy (c) and a handle without its tables: the
+    // full node step, one configuration (128 x 8).  A hop cap of the caller's needs no route of its
     // own: a lean walk makes the full step's hops one by one and hands a node that
     // reaches the cap outside its triangle to the full step (no jump table then; a
     // 2048^2-node swirl of 20 steps under a cap it never meets: 6.31 ms in the full
     // step, 4.40 here)
     const bool ext = a.exclude || a.order || a.grid_M > 0 || a.keep_t0;
-    if (stats || debug || a.order) {
-        if (ext) launch_f32_cfg<128, 8, true>(a, stats, debug, s);
+    if (stats || debug || a.order || !a.tri) {
+        if (ext || !(stats || debug)) launch_f32_cfg<128, 8, true>(a, stats, debug, s);
         else launch_f32_cfg<128, 8>(a, stats, debug, s);
         return;
     }

@@ -974,7 +974,7 @@ __device__ __forceinline__ void step_node(const FastArgs &a, int64_t i, int pi, 
     // node, is a point of the mesh alone, and its triangle is known (k_pair_tri;
     // without kLean it is walked to, as under a hop cap of the caller's, which
     // the way there from a far T^0 has to keep to).
-    const int32_t known = kLean && a.lean_moves > 0 && foot_on_pair(a.xyq[i], X, Y) ? a.pair_tri[i] : -1;
+    const int32_t known = kLean && a.lean_moves > 0 && a.pair_tri && foot_on_pair(a.xyq[i], X, Y) ? a.pair_tri[i] : -1;
     bool ids = true;           // w0..w2 are the vertex ids of the current triangle
     const uint32_t cap = (uint32_t)a.walk_cap;
     uint32_t &hops = c.hops;
@@ -1386,7 +1386,7 @@ inline void launch_fast_df_form(const FastArgs &a, bool stats, bool debug, unsig
         else launch_step_kernel(k_step_fast_df<true, false, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
     } else {
         if (debug) launch_step_kernel(k_step_fast_df<false, true, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
-        else if constexpr (kExt)    // strategy (c), a hop cap; the lean kernel takes the others
+        else if constexpr (kExt)    // strategy (c), no room for the lean kernel's tables
             launch_step_kernel(k_step_fast_df<false, false, kBlock, kMinBlocks, kExt, kCompact>, grid, kBlock, s, a);
     }
 }

@@ -265,3 +265,84 @@ def test_the_first_steady_run_of_a_handle_allocates_nothing(steps, precision):
     names = kernels_of(lambda: sl.sl_run(g.h, g.probs, 1, steps, v, w))
     assert any("k_apply" in n for n in names)
     assert g.torch.cuda.mem_get_info()[0] >= before - (4 << 20)
+
+
+# Steps and runs of every route, their values and T0, and the device memory of a
+# handle per node; with a library given, that one's.
+WITHOUT_TABLES = """
+import sys
+import numpy as np
+import torch
+import paper_2104_09189_gb300 as sl
+import sl_inputs as si
+if len(sys.argv) > 2:
+    sl._LIB_PATH = sys.argv[2]
+out = {}
+m = si.grid_mesh(90, 0.25, 3)
+c = si.courant_grid(64)
+for prec, dt in ((sl.SL_FP64, torch.float64), (sl.SL_FP32, torch.float32)):
+    for name, mesh, f, opts in (("b", m, si.swirl_field(), {}), ("steady", m, si.rotation_field(), {}),
+                                ("split", m, si.rotation_field(), {sl.SL_OPT_SPLIT: 1}),
+                                ("cap", m, si.swirl_field(), {sl.SL_OPT_WALK_CAP: 40}),
+                                ("a", m, si.swirl_field(), {sl.SL_OPT_STRATEGY: 1}),
+                                ("direct", c, si.swirl_field(), {sl.SL_OPT_STRATEGY: 2}),
+                                ("exclude", m, si.rotation_field(), {sl.SL_OPT_OUTSIDE: 1})):
+        h = sl.sl_mesh_create(*sl.pack_meshes([(mesh.xy, mesh.tri)] * 2 if name != "direct" else [(mesh.xy, mesh.tri)]),
+                              precision=prec)
+        np_ = sl.sl_mesh_info(h)["n_problems"]
+        probs = sl.problems([(f.kind, 0.05, f.packed())] * np_)
+        for o, x in opts.items():
+            sl.sl_mesh_set_option(h, o, x)
+        v = torch.tensor(np.tile(si.gaussian(mesh.xy), np_), dtype=dt, device="cuda")
+        w = torch.empty_like(v)
+        for r in range(2):
+            sl.sl_run(h, probs, 0, 3, v, w)
+            sl.sl_run(h, probs, 3, 7, v, w)
+            sl.sl_step(h, probs, 9, v, w)
+            t0 = torch.empty(v.numel(), dtype=torch.int32, device="cuda")
+            sl.sl_mesh_get_t0(h, t0)
+            out[f"{name} {prec} {r} v"] = w.cpu().numpy()
+            out[f"{name} {prec} {r} t0"] = t0.cpu().numpy()
+            sl.sl_mesh_reset_t0(h)
+        sl.sl_mesh_destroy(h)
+m = si.courant_grid(1000)
+before = torch.cuda.mem_get_info()[0]
+h = sl.sl_mesh_create(*sl.pack_meshes([(m.xy, m.tri)]))
+out["bytes"] = np.array((before - torch.cuda.mem_get_info()[0]) / m.n_nodes)
+np.savez(sys.argv[1], **out)
+"""
+
+
+def test_a_device_without_room_for_the_tables(tmp_path):
+    """A handle takes the tables and weights of the lean steps where memory is left
+    over; without them it is as small as its mesh and every step is the full one,
+    with the same results."""
+    import glob
+    import os
+    import subprocess
+    import sys
+
+    from paper_2104_09189_gb300 import _build
+    obj, lib = str(tmp_path / "api_device.o"), str(tmp_path / "libslwalk_small.so")
+    nvcc = [_build._nvcc(), *_build.ARCH]
+    subprocess.run([*nvcc, "-DSL_SPARE_BYTES=(1ull<<40)", "-O1", "-std=c++17", "-Xcompiler", "-fPIC", "-I", _build.INCLUDE,
+                    "-c", os.path.join(_build.CSRC, "api_device.cu"), "-o", obj], check=True)
+    others = [o for o in glob.glob(os.path.join(_build.BUILD, "*.o")) if "api_device" not in o]
+    subprocess.run([*nvcc, "-shared", "-o", lib, obj, *others, "-lpthread"], check=True)
+    got = []
+    for args in ((), (lib,)):
+        out = str(tmp_path / f"out{len(got)}.npz")
+        subprocess.run([sys.executable, "-c", WITHOUT_TABLES, out, *args], check=True, cwd=os.path.dirname(_build.INCLUDE))
+        got.append(np.load(out))
+    full, small = got
+    # xy 16, xyq 16, xyh 8, tv and tn 48, he 96, t0 8, t0v 16; allocations come in 2 MiB
+    assert float(small["bytes"]) <= 208 + 14 * 2.2 < float(full["bytes"])
+    for k in full.files:
+        if k == "bytes":
+            continue
+        if k.startswith(f"steady {sl.SL_FP64}") and k.endswith("v"):
+            assert np.abs(full[k] - small[k]).max() <= 11 * 2.0 ** -43, k     # the weights' values
+        elif k.startswith(f"split {sl.SL_FP64}") and k.endswith("v"):
+            assert np.abs(full[k] - small[k]).max() <= 11 * 2.0 ** -43, k
+        else:
+            assert np.array_equal(full[k], small[k]), k
