@@ -777,9 +777,10 @@ static sl_status launch_steady(sl_mesh *m, const FastArgs &a, int config, int32_
 static sl_status check_not_capturing(cudaStream_t s)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    SL_CUDA(cudaStreamIsCapturing(s, &st));
-    if (st != cudaStreamCaptureStatusNone) return fail(SL_E_CUDA, "the stream is being captured (use sl_step_noalloc)");
-    return SL_OK;
+    const cudaError_t e = cudaStreamIsCapturing(s, &st);
+    if (e == cudaSuccess && st == cudaStreamCaptureStatusNone) return SL_OK;
+    cudaGetLastError();     // (an error: the legacy stream while another one is captured)
+    return fail(SL_E_CUDA, "the stream is being captured (use sl_step_noalloc)");
 }
 
 static sl_status check_device(const sl_mesh *m)
@@ -852,7 +853,12 @@ static bool ensure_weights(sl_mesh *m)
 // are.  Storing costs about half a later step's time once and saves a third of
 // one per step, so runs of fewer than 4 steps go without; so do the counting
 // variants, the paper's experiments, split steps of a batch that is only
-// partly steady, and a device without room for the weights.
+// partly steady, and a device without room for the weights.  The settle pass has
+// no weights, and SL_OPT_SPLIT is the caller's choice or the tuner's, which weighs
+// steps that locate: split against fused with weights, 1.2 M nodes, 50 steps, a
+// third of them steady: 1.25 and 1.30 ms where feet move a third of a cell, 1.77 and
+// 1.63 at 3 cells, 4.02 and 2.39 at 20; three quarters steady 1.20 and 0.87 at a
+// third of a cell.  The tuner chose fused in each.
 constexpr int32_t kSteadySteps = 4;
 static bool mark_steady(sl_mesh *m, int32_t n_steps, bool split_rest, std::vector<FastProb> &fh)
 {

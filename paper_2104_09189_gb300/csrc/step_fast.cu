@@ -81,10 +81,11 @@ void launch_finish_df(const FastArgs &a, bool stats, bool debug, int sms, cudaSt
 //
 // They are configurations of the lean kernel.  Statistics, debug outputs,
 // strategy (c) and a handle without its tables (a.tri) run the full node step in
-// one configuration of its own.  A hop
-// cap of the caller's holds in the lean kernel too: its hops are the full step's
-// and end at the cap (a 1024^2-node swirl of 20 steps under a cap it never meets:
-// 1.33 ms in the full step, 1.22 here).
+// one configuration of its own.  A hop cap of the caller's holds in the lean
+// kernel too: its hops are the full step's and end at the cap (a 1024^2-node swirl
+// of 20 steps under a cap it never meets: 2.67 ms in the full step alone, 1.36
+// here; 1.22 if the feet at their nodes were sent to the triangle known for them,
+// past the walk that the cap is about).
 void launch_fast_df(const FastArgs &a, bool stats, bool debug, int config, cudaStream_t s)
 {
     if (stats || debug || a.order || !a.tri) {
@@ -395,7 +396,8 @@ __global__ void k_jump_fill(JumpBuildArgs a, int r, int from)
 
 // Pass 3: from the seed triangle, cross the edge the cell's centre lies
 // furthest beyond, at most 64 times (float: any triangle is a valid start).
-// A cell that found no seed takes triangle of its problem's first node.
+// A cell that found no seed takes the initial triangle of its problem's first
+// node.
 __global__ void k_jump_walk(JumpBuildArgs a, int from)
 {
     for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < a.cells; c += gridDim.x * blockDim.x) {

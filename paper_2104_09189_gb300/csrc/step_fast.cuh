@@ -29,7 +29,7 @@ struct FastProb {
     int32_t jump_g;     // cells per side of the problem's jump table
     int32_t jump_off;   // its first cell in FastArgs::jump
     float2 c[6];        // (hi, lo)
-    float2 dc;          // how far a foot moves from one step to this one (foot_moves): table fields the
+    float2 dc;          // how far a foot moves from one step to this one (jump_moves): table fields the
                         // change of c0 and c1, AFFINE the change of c0 and c3 (both within 2^-20)
 };
 
@@ -134,13 +134,16 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 // vertex of a triangle that does not hold it, is more than kJumpFar cells
 // away, so that the table's triangle is surely nearer.  A walk makes about two
 // hops per cell of the mesh, a cell of the table is two of the mesh wide, and
-// a jump costs two dependent gathers before its one or two hops: with 1, 2, 4
-// and 8 cells a study run of 150 k nodes with 4 hops per node took 422, 389,
+// a jump costs two dependent gathers before its one or two hops.  Alone, with 1,
+// 2, 4 and 8 cells, a study run of 150 k nodes with 4 hops per node took 422, 389,
 // 384 and 448 us, an FP32 swirl on 4.2 M nodes with 20 to 40 hops 3.17, 3.14,
-// 3.25 and 3.72 ms, and shorter walks stayed level from 2 on.  Four times the
-// cells gained 2 % there and nothing elsewhere.  From the initial triangles, a
-// rotation 360 cells long on 16.8 M nodes: 16.8 ms per run of 50 steps by
-// walking, 9.6 ms with the table (its first step 8.0 -> 0.7 ms).
+// 3.25 and 3.72 ms, and shorter walks stayed level from 2 on: 3 lies between the
+// two best.  With jump_moves below, which sends most far feet there first, 2, 3,
+// 4 and 8 are level (that swirl 2.37 to 2.38 ms, a batch of 2.8 M nodes 3.59) and 1
+// is slower (2.44, 3.67 ms).  Four times the cells gained 2 % on the swirl and
+// nothing elsewhere.  From the initial triangles, a rotation 360 cells long on
+// 16.8 M nodes: 16.8 ms per run of 50 steps by walking, 9.6 ms with the table (its
+// first step 8.0 -> 0.7 ms).
 constexpr float kJumpFar = 3.0f;
 __device__ __forceinline__ bool jump_far(float dx, float dy, const FastProb &P)
 {
